@@ -90,18 +90,21 @@ __device__ __forceinline__ void dep_trigger() { asm volatile("griddepcontrol.lau
 // Host: one launch.  `cooperative` asks for the co-residency guarantee; with ctx->overlap the
 // launch carries the programmatic attribute instead (the two cannot be combined), and co-residency
 // rests on the grid being one block per SM on a GPU that runs nothing else (a block that waits in
-// vain gives up after its spin limit and reports SPARK_ERR_TIMEOUT).
+// vain gives up after its spin limit and reports SPARK_ERR_TIMEOUT).  `chained`: the kernel ahead in the stream belongs to the
+// same call and writes nothing that this one touches before its dep_wait(), so the programmatic attribute is in place whatever
+// the context's setting (the first kernel of the call starts after everything before the call, and none of a chain's kernels
+// waits on other blocks).
 inline cudaError_t launch_kernel(const spark_ctx* ctx, const void* kern, unsigned grid, unsigned block, size_t smem,
-                                 cudaStream_t stream, bool cooperative, void** args) {
+                                 cudaStream_t stream, bool cooperative, void** args, bool chained = false) {
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(grid);
     cfg.blockDim = dim3(block);
     cfg.dynamicSmemBytes = smem;
     cfg.stream = stream;
-    cudaLaunchAttribute attr[1];
+    cudaLaunchAttribute attr[2];
     cfg.attrs = attr;
     cfg.numAttrs = 0;
-    if (ctx->overlap) {
+    if (ctx->overlap || chained) {
         attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
         attr[0].val.programmaticStreamSerializationAllowed = 1;
         cfg.numAttrs = 1;
@@ -109,6 +112,16 @@ inline cudaError_t launch_kernel(const spark_ctx* ctx, const void* kern, unsigne
         attr[0].id = cudaLaunchAttributeCooperative;
         attr[0].val.cooperative = 1;
         cfg.numAttrs = 1;
+    }
+    // The kernels of 512 threads take their weights and cache rows through registers, and loads in flight live in L1 lines (up to
+    // 64 KB a block).  Left alone an SM keeps the split of L1 and shared memory that the kernel ahead needed: behind a tensor-core
+    // kernel with 160 to 227 KB of stages that leaves 28 to 60 KB of L1, and the 2B attention at batch 8 took 36 instead of 27 us
+    // (9B layer at batch 8: 126.8 -> 112.9 us with half and half; batch 1: 58.1 -> 55.0).  One split for all of them, because
+    // changing it needs an idle SM (the smallest split that fits each kernel: 2B layer at batch 1 +0.2 us); not for the small
+    // helper kernels between tensor-core kernels for the same reason (2B layer, batch 8: +1.5 us).
+    if (block == 512 && smem >= 8192) {
+        attr[cfg.numAttrs].id = cudaLaunchAttributePreferredSharedMemoryCarveout;
+        attr[cfg.numAttrs++].val.sharedMemCarveout = 50;     // percent; raised by the driver to what the kernel needs
     }
     return cudaLaunchKernelExC(&cfg, kern, args);
 }

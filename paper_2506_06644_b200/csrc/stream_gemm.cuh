@@ -1,0 +1,215 @@
+// The weight-streaming GEMM of the token-chunk kernels (tcgen05): D[rows][tokens] = A[rows][K] . X[tokens][K]^T for up to
+// 64 tokens, A a bf16 weight matrix that is read once, X the fp32 activations as two bf16 terms (hi rows, then lo rows).
+//
+// What bounds it is the weight stream, so the split of the work is by bytes: the (tile, K chunk) pairs of all tiles form one
+// sequence, tile after tile, and every block takes a contiguous part of it, whatever the number of tiles.  A tile that falls to
+// several blocks is completed by the caller's epilogue (reductions into an initialised output).  Per block: warp 0 moves
+// 64-element K chunks of A (128 rows) and X (both terms in one box) with TMA through a ring of stages, warp 1 issues the MMAs and
+// four epilogue warps drain one of two accumulator sets while the next segment runs.  Both terms are one operand tile of
+// N = 2 x tokens, so the weight tile is read from shared memory once.  The weights do not depend on the kernel ahead: their first
+// stages are requested before griddepcontrol.wait.  Bounded waits as in tc_common.cuh.
+// Measured, 64 tokens, 256000 x 2304: 201 us = 5.9 TB/s (0.90 of the measured copy rate); 17 tokens 182 us (0.99).
+#pragma once
+
+#include "tc_common.cuh"
+
+namespace spark {
+namespace tc {
+
+constexpr int kStreamMaxStages = 8;
+constexpr int kStreamRows = 128;
+constexpr int kStreamTileBytes = kStreamRows * kChunk * 2;
+
+struct StreamShared {
+    unsigned long long full[kStreamMaxStages], empty[kStreamMaxStages];
+    unsigned long long acc_full[2], acc_empty[2];
+    uint32_t tmem;
+    int abort_flag;
+};
+
+struct StreamPlan {
+    int total;               // K chunks of all tiles
+    int grid, per;           // blocks; chunks a block takes (0: equal parts of the sequence or of each tile)
+    int part, rem;           // an equal part is `part` chunks, one more for the first `rem` of them (of the sequence, or of a tile)
+    int split;               // every tile is cut into this many pieces (0: no such regular cut)
+    int call;                // K chunks of a tile
+    int ntok;                // tokens rounded up to a multiple of 16: half of the MMAs' N; X has rows term * ntok + token
+    int stages;
+    int stage_bytes;
+    uint32_t tmem_cols;
+};
+
+// Start of a block's part of the sequence (no 64-bit division: it sits in front of the first load).
+__host__ __device__ inline int stream_begin(const StreamPlan& sp, int block) {
+    if (sp.per > 0) return block < sp.grid ? block * sp.per : sp.total;
+    if (sp.split > 0) {
+        const int tile = block / sp.split, i = block - tile * sp.split;
+        return tile * sp.call + i * sp.part + (i < sp.rem ? i : sp.rem);
+    }
+    return block * sp.part + (block < sp.rem ? block : sp.rem);
+}
+
+// Host: fills in the plan for at most `smem_limit` bytes of dynamic shared memory.  False: does not fit.
+inline bool stream_plan(StreamPlan& sp, int sms, int tiles, int call, int tokens, size_t smem_limit) {
+    sp.call = call;
+    sp.total = tiles * call;
+    sp.per = sp.split = 0;
+    // A piece of a tile costs its block an epilogue (1.5 to 4 us with the reductions of 16 to 64 tokens), so blocks get one piece
+    // of one tile, or whole tiles, where that leaves 0.6 / 0.9 of the SMs busy: fewer SMs still draw what HBM gives (4096 x 2304,
+    // 64 tokens: 128 blocks of one piece 9.7 us, 148 equal parts of two pieces each 15.4 us).  Otherwise equal parts.
+    const int ks = sms / tiles < call ? sms / tiles : call, m = (tiles + sms - 1) / sms;
+    if (ks >= 1 && (tiles * ks * 10 >= sms * 6 || ks == call)) {
+        sp.split = ks;
+        sp.grid = tiles * ks;
+    } else if (tiles > sms && m <= 4 && (tiles + m - 1) / m * 10 >= sms * 9) {
+        sp.per = m * call;
+        sp.grid = (tiles + m - 1) / m;
+    } else {
+        sp.grid = sp.total < sms ? sp.total : sms;
+    }
+    const int of = sp.split > 0 ? call : sp.total, by = sp.split > 0 ? sp.split : sp.grid;
+    sp.part = of / by;
+    sp.rem = of % by;
+    sp.ntok = (tokens + 15) & ~15;
+    sp.stage_bytes = kStreamTileBytes + 2 * sp.ntok * kChunk * 2;
+    const int fit = static_cast<int>((smem_limit - 1024) / sp.stage_bytes);
+    // more than eight stages (128 KB of weights in flight per SM, three times what the latency of HBM needs) only delays the
+    // small loads of the kernel ahead that queue behind them
+    sp.stages = fit < kStreamMaxStages ? fit : kStreamMaxStages;
+    uint32_t cols = 32;
+    while (cols < static_cast<uint32_t>(4 * sp.ntok)) cols *= 2;
+    sp.tmem_cols = cols;
+    return sp.stages >= 2 && cols <= 512 && tiles > 0 && call > 0;
+}
+inline size_t stream_smem(const StreamPlan& sp) { return static_cast<size_t>(sp.stages) * sp.stage_bytes + 1024; }
+
+// One block's work.  epi(tile, whole, row, n0, v): sixteen tokens' values of one row (0..127) of a tile; `whole`: the block holds
+// all of the tile's K range.
+template <class Epi>
+__device__ __forceinline__ void stream_gemm(const StreamPlan& sp, StreamShared& sh, unsigned char* raw, const CUtensorMap* map_w,
+                                            const CUtensorMap* map_x, WsHeader* hdr, Epi epi) {
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int p0 = stream_begin(sp, blockIdx.x), p1 = stream_begin(sp, blockIdx.x + 1), n = p1 - p0;
+    const uint32_t xbytes = static_cast<uint32_t>(2 * sp.ntok) * (kChunk * 2);
+    const int stages = sp.stages;
+    if (tid == 0) {
+        for (int s = 0; s < stages; ++s) {
+            mbar_init(smem_addr(&sh.full[s]), 1u);
+            mbar_init(smem_addr(&sh.empty[s]), 1u);
+        }
+        for (int b = 0; b < 2; ++b) {
+            mbar_init(smem_addr(&sh.acc_full[b]), 1u);
+            mbar_init(smem_addr(&sh.acc_empty[b]), 4u);
+        }
+        sh.abort_flag = 0;
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+    }
+    if (warp == 1) tmem_alloc(smem_addr(&sh.tmem), sp.tmem_cols);
+    tc_fence_before();
+    __syncthreads();
+    tc_fence_after();
+    const uint32_t base = (smem_addr(raw) + 1023u) & ~1023u;
+    const uint32_t tmem = sh.tmem;
+    volatile int* abort_flag = &sh.abort_flag;
+    dep_trigger();           // the kernel behind only requests its weights before it waits for this one
+
+    if (warp == 0) {
+        if (lane == 0) {
+            int tile = p0 / sp.call, c = p0 - tile * sp.call, cx = c;
+            const int pre = min(n, stages);
+            for (int i = 0; i < pre; ++i) {
+                const uint32_t bar = smem_addr(&sh.full[i]);
+                mbar_expect_tx(bar, kStreamTileBytes + xbytes);
+                tma_load_2d(base + i * sp.stage_bytes, map_w, bar, c * kChunk, tile * kStreamRows);
+                if (++c == sp.call) { c = 0; ++tile; }
+            }
+            dep_wait();
+            for (int i = 0; i < pre; ++i) {
+                tma_load_2d(base + i * sp.stage_bytes + kStreamTileBytes, map_x, smem_addr(&sh.full[i]), cx * kChunk, 0);
+                if (++cx == sp.call) cx = 0;
+            }
+            int s = 0, issued = pre;
+            uint32_t parity = 0u;
+            for (int i = pre; i < n; ++i) {
+                if (!mbar_wait(smem_addr(&sh.empty[s]), parity, abort_flag)) break;
+                const uint32_t bar = smem_addr(&sh.full[s]), dst = base + s * sp.stage_bytes;
+                mbar_expect_tx(bar, kStreamTileBytes + xbytes);
+                tma_load_2d(dst, map_w, bar, c * kChunk, tile * kStreamRows);
+                tma_load_2d(dst + kStreamTileBytes, map_x, bar, c * kChunk, 0);
+                if (++c == sp.call) { c = 0; ++tile; }
+                if (++s == stages) { s = 0; parity ^= 1u; }
+                issued = i + 1;
+            }
+            if (*abort_flag != 0) {      // the copies in flight land (bounded) before the block goes
+                for (int i = max(0, issued - stages); i < issued; ++i) {
+                    const long long t0 = clock64();
+                    while (!mbar_try(smem_addr(&sh.full[i % stages]), static_cast<uint32_t>(i / stages) & 1u))
+                        if (clock64() - t0 > kTcSpinLimit) break;
+                }
+            }
+        }
+    } else if (warp == 1) {
+        // the whole warp walks the loop; one elected lane issues
+        const uint32_t elected = elect_lane(), idesc = instr_desc(128, 2 * sp.ntok, false);
+        int s = 0, pos = p0, seg = 0;
+        uint32_t parity = 0u;
+        bool ok = true;
+        while (pos < p1 && ok) {
+            const int end = min(p1, (pos / sp.call + 1) * sp.call), b = seg & 1;
+            if (seg >= 2) ok = __all_sync(kFull, mbar_wait(smem_addr(&sh.acc_empty[b]), ((seg >> 1) & 1) ^ 1, abort_flag));
+            const uint32_t acc = tmem + static_cast<uint32_t>(b * 2 * sp.ntok);
+            tc_fence_after();
+            for (uint32_t more = 0u; pos < end && ok; ++pos, more = 1u) {
+                ok = __all_sync(kFull, mbar_wait(smem_addr(&sh.full[s]), parity, abort_flag));
+                if (!ok) break;
+                tc_fence_after();
+                const uint32_t a0 = base + s * sp.stage_bytes;
+                const uint64_t ad = smem_desc(a0, 0u, 1024u), xd = smem_desc(a0 + kStreamTileBytes, 0u, 1024u);
+#pragma unroll
+                for (int j = 0; j < kChunk / 16; ++j)      // descriptors count in 16-byte units
+                    umma_bf16_elected(acc, ad + 2 * j, xd + 2 * j, idesc, j == 0 ? more : 1u, elected);
+                umma_commit_elected(smem_addr(&sh.empty[s]), elected);
+                if (++s == stages) { s = 0; parity ^= 1u; }
+            }
+            if (ok) umma_commit_elected(smem_addr(&sh.acc_full[b]), elected);
+            ++seg;
+        }
+    } else {
+        const int q = warp & 3;                                    // tensor-memory lanes 32 q .. 32 q + 31
+        dep_wait();
+        int pos = p0, seg = 0;
+        while (pos < p1) {
+            const int tile = pos / sp.call, end = min(p1, (tile + 1) * sp.call), b = seg & 1;
+            if (!__all_sync(kFull, mbar_wait(smem_addr(&sh.acc_full[b]), (seg >> 1) & 1, abort_flag))) break;      // warp-uniform: tcgen05.ld is warp-wide
+            tc_fence_after();
+            const uint32_t taddr = tmem + static_cast<uint32_t>(b * 2 * sp.ntok) + (static_cast<uint32_t>(q * 32) << 16);
+            for (int n0 = 0; n0 < sp.ntok; n0 += 16) {
+                float v[16];
+                tmem_ld16_sum(taddr + n0, taddr + sp.ntok + n0, v);
+                epi(tile, end - pos == sp.call, q * 32 + lane, n0, v);
+            }
+            tc_fence_before();
+            __syncwarp();
+            if (lane == 0) asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_addr(&sh.acc_empty[b])) : "memory");
+            pos = end;
+            ++seg;
+        }
+    }
+    tc_fence_before();
+    __syncthreads();
+    if (warp == 1) {
+        tc_fence_after();
+        tmem_free(tmem, sp.tmem_cols);
+    }
+    if (tid == 0 && sh.abort_flag != 0) atomicCAS(&hdr->status, SPARK_OK, SPARK_ERR_TIMEOUT);
+}
+
+// The two bf16 terms of an fp32 value pair: x = hi + lo, 16 significant bits.
+__device__ __forceinline__ void split_pair(float a, float b, unsigned& hi, unsigned& lo) {
+    hi = pack2_bf16(a, b);
+    lo = pack2_bf16(a - __uint_as_float(hi << 16), b - __uint_as_float(hi & 0xffff0000u));
+}
+
+}  // namespace tc
+}  // namespace spark
