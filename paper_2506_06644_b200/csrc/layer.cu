@@ -775,6 +775,18 @@ __global__ void chunk_lengths_kernel(int32_t* len, int n, int first) {      // l
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i < n) len[i] = first + i;
 }
+
+int prefill_spans(spark_ctx* ctx, const spark_layer_weights* w, const spark_layer_cfg* cfg, const spark_kv_cache* cache, int64_t n_layers, float* h,
+                  int64_t n_tokens, int64_t start, int64_t span, cudaStream_t st) {
+    for (int64_t c0 = 0; c0 < n_tokens; c0 += span) {
+        const int64_t T = n_tokens - c0 < span ? n_tokens - c0 : span;
+        for (int64_t l = 0; l < n_layers; ++l) {
+            const int rc = span_layer_launch(ctx, w + l, cfg + l, cache + l, h + c0 * cfg[0].d, T, start + c0, st);
+            if (rc != SPARK_OK) return rc;
+        }
+    }
+    return SPARK_OK;
+}
 }  // namespace
 
 extern "C" int spark_prefill(spark_ctx* ctx, const spark_layer_weights* w, const spark_layer_cfg* cfg, const spark_kv_cache* cache,
@@ -789,6 +801,8 @@ extern "C" int spark_prefill(spark_ctx* ctx, const spark_layer_weights* w, const
     }
     if (!on_device(ctx)) return SPARK_ERR_INVALID_ARG;
     cudaStream_t st = static_cast<cudaStream_t>(stream);
+    // as many tokens at a time as the workspace holds, when the layers allow it (span.cu)
+    if (const int64_t span = span_tokens(ctx, w, cfg, cache, n_layers, h, n_tokens, start)) return prefill_spans(ctx, w, cfg, cache, n_layers, h, n_tokens, start, span, st);
     for (int64_t c0 = 0; c0 < n_tokens; c0 += chunk) {
         const int64_t T = n_tokens - c0 < chunk ? n_tokens - c0 : chunk;
         int n = static_cast<int>(T), first = static_cast<int>(start + c0 + 1);
@@ -833,6 +847,9 @@ extern "C" int spark_prefill_pipelined(spark_ctx* const* ctxs, float* const* scr
     if (!on_device(ctxs[0])) return SPARK_ERR_INVALID_ARG;
     cudaStream_t st[kMaxInflight];
     for (int i = 0; i < n; ++i) st[i] = static_cast<cudaStream_t>(streams[i]);
+    // spans fill the GPU by themselves: they run on the first context and stream, where the call forks from and joins
+    if (const int64_t span = span_tokens(ctxs[0], w, cfg, cache, n_layers, h, n_tokens, start))
+        return prefill_spans(ctxs[0], w, cfg, cache, n_layers, h, n_tokens, start, span, st[0]);
     // done[s][l]: layer l of the newest chunk on stream s has finished; fork and join around the call
     const size_t n_ev = static_cast<size_t>(n) * static_cast<size_t>(n_layers) + 1 + static_cast<size_t>(n);
     cudaEvent_t* ev = new (std::nothrow) cudaEvent_t[n_ev];
