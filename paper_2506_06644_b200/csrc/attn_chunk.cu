@@ -36,10 +36,7 @@ struct ChunkParams {
     const int32_t* ctx_len;    // [T]
     const double* zs_in;       // nullable: Q(1 - k_attn / L_t) per token from an earlier kernel
     int T, n_q, n_kv, gq, hd, r, window, k_attn;
-    // The queries are taken in sub-chunks of `tps` tokens (tps * gq <= kColMax columns per KV head); KV head g of sub-chunk s is
-    // the "virtual head" s * n_kv + g, which has columns, operand rows and score columns of its own and reads cache g.
-    int tps, nsub;
-    int ncol, ncolp;           // columns of a full sub-chunk: tps * gq, rounded up to a multiple of 16
+    int ncol, ncolp;           // T * gq, rounded up to a multiple of 16
     int64_t cap;
     float* o;                  // [T][n_q][hd], normalised
     float* lsum;               // nullable: [T][n_q] = 1 (0 for an empty selection): the caller divides by it
@@ -48,20 +45,18 @@ struct ChunkParams {
     // workspace
     double* zt;                // [T]
     int* range;                // [T][2] = lo_t, n_t
-    __nv_bfloat16* qhi;        // [virtual heads][kColMax][r]
+    __nv_bfloat16* qhi;        // [n_kv][kColMax][r]
     __nv_bfloat16* qlo;
-    float* S;                  // [virtual heads][kColMax][scap]
+    float* S;                  // [n_kv][kColMax][scap]
     int64_t scap;              // column stride of S: cap + 32, so that the columns' lines do not all fall on the same slices
     // dense second stage (masked weights x value rows on the tensor cores) only
-    __nv_bfloat16* q2hi;       // [virtual heads][kColMax][hd - r]: the gate's query part as two bf16 terms
+    __nv_bfloat16* q2hi;       // [n_kv][kColMax][hd - r]: the gate's query part as two bf16 terms
     __nv_bfloat16* q2lo;
-    float4* colinfo;           // [virtual heads][kColMax] = theta, maximum of the survivors' scores, lo, n (the last two as int bits)
+    float4* colinfo;           // [n_kv][kColMax] = theta, maximum of the survivors' scores, lo, n (the last two as int bits)
     float* zsum;               // [T][n_q] sum of exp(s - max) over the survivors
     int dense;
     WsHeader* hdr;
 };
-
-__device__ __forceinline__ int sub_tokens(const ChunkParams& p, int sub) { return min(p.tps, p.T - sub * p.tps); }
 
 __device__ __forceinline__ void token_range(const ChunkParams& p, int t, int& lo, int& n) {
     n = p.ctx_len[t];
@@ -117,15 +112,12 @@ constexpr int kChunkBBytes = 2 * 2 * kColMax * kChunk * 2;   // per K chunk: hi 
 constexpr int kChunkStageBytes = kChunkABytes + kChunkBBytes;
 constexpr uint32_t kChunkCols = 512;                         // two accumulators of 128 rows x (hi | lo) columns
 
-constexpr int kMaxSub = 128;
-
 struct ChunkShared {
     unsigned long long full[kChunkStages], empty[kChunkStages];
     unsigned long long acc_full[2], acc_empty[2];
     uint32_t tmem;
     int abort_flag;
-    int tiles[kMaxSub + 1];      // row tiles of all virtual heads of the sub-chunks before this one
-    int first[kMaxSub], rows[kMaxSub];      // a sub-chunk's first row tile; end of the rows that its tokens see
+    int n_max;
 };
 constexpr int kChunkThreads = 64 + 8 * 32;      // warp 0: TMA, warp 1: MMA + tensor memory, warps 2..9: epilogue
 
@@ -135,7 +127,7 @@ attn_chunk_scores_kernel(const ChunkParams p, const __grid_constant__ CUtensorMa
     extern __shared__ unsigned char tc_raw[];
     __shared__ ChunkShared sh;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    const int nkc = (p.r + kChunk - 1) / kChunk;      // a last chunk that is not full arrives padded with zeros
+    const int nkc = p.r / kChunk;
     if (tid == 0) {
         for (int s = 0; s < kChunkStages; ++s) {
             mbar_init(smem_addr(&sh.full[s]), 1u);
@@ -152,20 +144,10 @@ attn_chunk_scores_kernel(const ChunkParams p, const __grid_constant__ CUtensorMa
     if (warp == 1) tmem_alloc(smem_addr(&sh.tmem), kChunkCols);
     dep_wait();                  // everything this kernel reads comes from the kernels ahead (cache rows, queries, ranges)
     dep_trigger();
-    for (int sub = tid; sub < p.nsub; sub += kChunkThreads) {
-        int m = 1, lo = 0x7fffffff;
-        for (int t = sub * p.tps, e = t + sub_tokens(p, sub); t < e; ++t) {
-            m = max(m, p.range[2 * t + 1]);
-            lo = min(lo, p.range[2 * t]);
-        }
-        sh.first[sub] = lo / 128;
-        sh.rows[sub] = m;
-        sh.tiles[sub + 1] = p.n_kv * ((m + 127) / 128 - lo / 128);
-    }
-    __syncthreads();
     if (tid == 0) {
-        sh.tiles[0] = 0;
-        for (int sub = 0; sub < p.nsub; ++sub) sh.tiles[sub + 1] += sh.tiles[sub];
+        int m = 1;
+        for (int t = 0; t < p.T; ++t) m = max(m, p.range[2 * t + 1]);
+        sh.n_max = m;
     }
     tc_fence_before();
     __syncthreads();
@@ -173,14 +155,8 @@ attn_chunk_scores_kernel(const ChunkParams p, const __grid_constant__ CUtensorMa
     const uint32_t base = (smem_addr(tc_raw) + 1023u) & ~1023u;
     const uint32_t tmem = sh.tmem;
     volatile int* abort_flag = &sh.abort_flag;
-    const int total = sh.tiles[p.nsub];
-    // tile number -> sub-chunk (advanced from the last one: tiles come in ascending order), KV head, row tile
-    auto locate = [&](int tile, int& sub, int& g, int& rb) {
-        while (tile >= sh.tiles[sub + 1]) ++sub;
-        const int per = (sh.tiles[sub + 1] - sh.tiles[sub]) / p.n_kv, i = tile - sh.tiles[sub];
-        g = i / per;
-        rb = sh.first[sub] + i - g * per;
-    };
+    const int n_max = sh.n_max;
+    const int tiles_h = (n_max + 127) / 128, total = p.n_kv * tiles_h;
     const int t0 = static_cast<int>(static_cast<int64_t>(blockIdx.x) * total / gridDim.x);
     const int t1 = static_cast<int>(static_cast<int64_t>(blockIdx.x + 1) * total / gridDim.x);
     const uint32_t qbytes = static_cast<uint32_t>(p.ncolp) * kChunk * 2;          // one term of one K chunk of the queries
@@ -191,20 +167,18 @@ attn_chunk_scores_kernel(const ChunkParams p, const __grid_constant__ CUtensorMa
             tma_prefetch_desc(&map_k1);
             tma_prefetch_desc(&map_qhi);
             tma_prefetch_desc(&map_qlo);
-            int issued = 0, sub = 0;
+            int issued = 0;
             for (int tile = t0; tile < t1; ++tile) {
                 const int i = tile - t0, s = i % kChunkStages;
                 if (i >= kChunkStages && !mbar_wait(smem_addr(&sh.empty[s]), ((i / kChunkStages) & 1) ^ 1, abort_flag)) break;
-                int g, rb;
-                locate(tile, sub, g, rb);
-                const int vrow = (sub * p.n_kv + g) * kColMax;
+                const int g = tile / tiles_h, rb = tile - g * tiles_h;
                 const uint32_t bar = smem_addr(&sh.full[s]), dst = base + s * kChunkStageBytes;
                 mbar_expect_tx(bar, stage_tx);
                 for (int kc = 0; kc < nkc; ++kc) {
                     tma_load_2d(dst + kc * (128 * kChunk * 2), &map_k1, bar, kc * kChunk, static_cast<int>(g * p.cap + rb * 128));
                     const uint32_t qd = dst + kChunkABytes + kc * (2 * kColMax * kChunk * 2);
-                    tma_load_2d(qd, &map_qhi, bar, kc * kChunk, vrow);
-                    tma_load_2d(qd + qbytes, &map_qlo, bar, kc * kChunk, vrow);    // lo rows right behind the hi rows
+                    tma_load_2d(qd, &map_qhi, bar, kc * kChunk, g * kColMax);
+                    tma_load_2d(qd + qbytes, &map_qlo, bar, kc * kChunk, g * kColMax);    // lo rows right behind the hi rows
                 }
                 issued = i + 1;
             }
@@ -238,29 +212,26 @@ attn_chunk_scores_kernel(const ChunkParams p, const __grid_constant__ CUtensorMa
         // eight warps: two per tensor-memory lane quadrant, each taking half of the columns
         const int q = warp & 3, half = (warp - 2) >> 2;
         bool ok = true;
-        int sub = 0;
         for (int tile = t0; tile < t1 && ok; ++tile) {
             const int i = tile - t0, b = i & 1;
-            int g, rb;
-            locate(tile, sub, g, rb);
-            const int ncol = sub_tokens(p, sub) * p.gq, n_max = sh.rows[sub];
+            const int g = tile / tiles_h, rb = tile - g * tiles_h;
             ok = __all_sync(kFull, mbar_wait(smem_addr(&sh.acc_full[b]), (i >> 1) & 1, abort_flag));
             if (!ok) break;
             tc_fence_after();
             const int j = rb * 128 + q * 32 + lane;
             const uint32_t tacc = tmem + b * 256 + (static_cast<uint32_t>(q * 32) << 16);
-            float* scol = p.S + static_cast<int64_t>(sub * p.n_kv + g) * kColMax * p.scap + j;
+            float* scol = p.S + static_cast<int64_t>(g) * kColMax * p.scap + j;
 #pragma unroll
             for (int cc = 0; cc < 2; ++cc) {
                 const int cb = 2 * half + cc;
-                if (cb * 32 < ncol) {
+                if (cb * 32 < p.ncol) {
                     float v[32], w[32];
                     tmem_ld32(tacc + cb * 32, v);
                     tmem_ld32(tacc + p.ncolp + cb * 32, w);
                     if (j < n_max) {
 #pragma unroll
                         for (int c = 0; c < 32; ++c)
-                            if (cb * 32 + c < ncol) scol[static_cast<int64_t>(cb * 32 + c) * p.scap] = v[c] + w[c];
+                            if (cb * 32 + c < p.ncol) scol[static_cast<int64_t>(cb * 32 + c) * p.scap] = v[c] + w[c];
                     }
                 }
             }
@@ -656,12 +627,11 @@ __global__ void __launch_bounds__(256, 4) attn_chunk_stats_kernel(const ChunkPar
     __shared__ float s_th, s_mx;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int t = blockIdx.x / p.n_q, h = blockIdx.x - t * p.n_q;
-    const int g = h / p.gq, sub = t / p.tps, col = (t - sub * p.tps) * p.gq + (h - g * p.gq);
-    const int64_t vcol = static_cast<int64_t>(sub * p.n_kv + g) * kColMax + col;      // column of the virtual head
+    const int g = h / p.gq, col = t * p.gq + (h - g * p.gq);
     dep_wait();
     dep_trigger();
     const int lo = p.range[2 * t], n = p.range[2 * t + 1], L = n - lo;
-    const float* scol = p.S + vcol * p.scap;
+    const float* scol = p.S + (static_cast<int64_t>(g) * kColMax + col) * p.scap;
     if (tid < p.hd) p.o[static_cast<int64_t>(blockIdx.x) * p.hd + tid] = 0.f;       // the dense kernel adds into it
     // The column's visible part stays in registers between the three sweeps: eight 16-byte loads per thread starting at the
     // 16-byte boundary at or below lo (rows outside [lo, n) read as -inf); longer columns are swept from L2 three times.
@@ -780,7 +750,7 @@ __global__ void __launch_bounds__(256, 4) attn_chunk_stats_kernel(const ChunkPar
         float z = 0.f;
 #pragma unroll
         for (int w = 0; w < 8; ++w) z += redf[w];
-        p.colinfo[vcol] = make_float4(th, mx, __int_as_float(lo), __int_as_float(n));
+        p.colinfo[g * kColMax + col] = make_float4(th, mx, __int_as_float(lo), __int_as_float(n));
         p.zsum[blockIdx.x] = total > 0 ? z : 0.f;
         if (p.lsum != nullptr) p.lsum[blockIdx.x] = total > 0 ? z : 0.f;
         if (p.theta != nullptr) p.theta[blockIdx.x] = th;
@@ -804,13 +774,11 @@ attn_chunk_dense_kernel(const ChunkParams p, const __grid_constant__ CUtensorMap
     extern __shared__ unsigned char tc_raw[];
     __shared__ DenseShared sh;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    const int d2 = p.hd - p.r, nk2 = (d2 + kChunk - 1) / kChunk, nvh = (p.hd + 127) / 128;      // partial boxes arrive padded with zeros
+    const int d2 = p.hd - p.r, nk2 = d2 / kChunk, nvh = p.hd / 128;
     const int ncg = (p.ncol + kDN - 1) / kDN;
     const int grp = blockIdx.x / nsplit, part = blockIdx.x - grp * nsplit;
-    // the last sub-chunks see the most rows: their groups come first
-    const int vh = p.nsub * p.n_kv - 1 - grp / ncg, cg = grp % ncg, sub = vh / p.n_kv, g = vh - sub * p.n_kv;
-    const int ncol = sub_tokens(p, sub) * p.gq, tok0 = sub * p.tps;
-    const int col0 = cg * kDN;                                  // first column of this block within the virtual head
+    const int g = grp / ncg, cg = grp - g * ncg;
+    const int col0 = cg * kDN;                                  // first column of this block within the KV head
     if (tid == 0) {
         for (int s = 0; s < kDSlots; ++s) {
             mbar_init(smem_addr(&sh.full[s]), 1u);
@@ -833,16 +801,16 @@ attn_chunk_dense_kernel(const ChunkParams p, const __grid_constant__ CUtensorMap
     dep_trigger();
     if (tid < kDN) {
         const int col = col0 + tid;
-        sh.info[tid] = col < ncol ? p.colinfo[vh * kColMax + col] : make_float4(INFINITY, 0.f, __int_as_float(0), __int_as_float(0));
+        sh.info[tid] = col < p.ncol ? p.colinfo[g * kColMax + col] : make_float4(INFINITY, 0.f, __int_as_float(0), __int_as_float(0));
         const int t = col / p.gq, h = g * p.gq + (col - t * p.gq);
-        sh.orow[tid] = col < ncol ? p.o + (static_cast<int64_t>(tok0 + t) * p.n_q + h) * p.hd : nullptr;
+        sh.orow[tid] = col < p.ncol ? p.o + (static_cast<int64_t>(t) * p.n_q + h) * p.hd : nullptr;
     }
     if (tid == 0) {
         // rows any of this block's columns may see, and the end of what the chunk has written
         int lo_min = 0x7fffffff, n_max = 0, n_all = 0, lo_max = 0, n_min = 0x7fffffff;
-        for (int t = p.nsub > 1 ? p.T - 1 : 0; t < p.T; ++t) n_all = max(n_all, p.range[2 * t + 1]);      // several sub-chunks: lengths ascend
-        const int c_end = min(ncol, col0 + kDN);
-        for (int t = tok0 + col0 / p.gq; t <= tok0 + (c_end - 1) / p.gq; ++t) {
+        for (int t = 0; t < p.T; ++t) n_all = max(n_all, p.range[2 * t + 1]);
+        const int c_end = min(p.ncol, col0 + kDN);
+        for (int t = col0 / p.gq; t <= (c_end - 1) / p.gq; ++t) {
             lo_min = min(lo_min, p.range[2 * t]);
             n_max = max(n_max, p.range[2 * t + 1]);
             lo_max = max(lo_max, p.range[2 * t]);
@@ -863,7 +831,7 @@ attn_chunk_dense_kernel(const ChunkParams p, const __grid_constant__ CUtensorMap
     unsigned char* ring_gen = tc_raw + (base - smem_addr(tc_raw));
     const uint32_t tmem = sh.tmem;
     volatile int* abort_flag = &sh.abort_flag;
-    const int tile_lo = col0 < ncol ? sh.lo_min / 128 : 0, tile_hi = (sh.n_max + 127) / 128, nt_all = max(0, tile_hi - tile_lo);
+    const int tile_lo = sh.lo_min / 128, tile_hi = (sh.n_max + 127) / 128, nt_all = max(0, tile_hi - tile_lo);
     const int ta = tile_lo + static_cast<int>(static_cast<int64_t>(part) * nt_all / nsplit);
     const int tb = tile_lo + static_cast<int>(static_cast<int64_t>(part + 1) * nt_all / nsplit);
     const int n = tb - ta;                                      // this block's tiles
@@ -878,8 +846,8 @@ attn_chunk_dense_kernel(const ChunkParams p, const __grid_constant__ CUtensorMap
                 const uint32_t bar = smem_addr(&sh.q_full);
                 mbar_expect_tx(bar, static_cast<uint32_t>(2 * nk2) * kDN * 128);
                 for (int kc = 0; kc < nk2; ++kc) {
-                    tma_load_2d(qbase + kc * (kDN * 128), &map_q2hi, bar, kc * kChunk, vh * kColMax + col0);
-                    tma_load_2d(qbase + (nk2 + kc) * (kDN * 128), &map_q2lo, bar, kc * kChunk, vh * kColMax + col0);
+                    tma_load_2d(qbase + kc * (kDN * 128), &map_q2hi, bar, kc * kChunk, g * kColMax + col0);
+                    tma_load_2d(qbase + (nk2 + kc) * (kDN * 128), &map_q2lo, bar, kc * kChunk, g * kColMax + col0);
                 }
             }
             int it = 0;
@@ -973,10 +941,10 @@ attn_chunk_dense_kernel(const ChunkParams p, const __grid_constant__ CUtensorMap
         float s1n[16];
         auto request_s1 = [&](int i) {
             const int tok = (ta + i) * 128 + row;
-            const float* srow = p.S + (static_cast<int64_t>(vh) * kColMax + col0 + cbase) * p.scap + tok;
+            const float* srow = p.S + (static_cast<int64_t>(g) * kColMax + col0 + cbase) * p.scap + tok;
 #pragma unroll
             for (int c = 0; c < 16; ++c)
-                s1n[c] = (tok < n_all && col0 + cbase + c < ncol) ? __ldcg(srow + static_cast<int64_t>(c) * p.scap) : -INFINITY;
+                s1n[c] = (tok < n_all && col0 + cbase + c < p.ncol) ? __ldcg(srow + static_cast<int64_t>(c) * p.scap) : -INFINITY;
         };
         request_s1(0);
         for (int i = 0; i < n && ok; ++i) {
@@ -1056,9 +1024,7 @@ attn_chunk_dense_kernel(const ChunkParams p, const __grid_constant__ CUtensorMap
 #pragma unroll
                 for (int c = 0; c < 16; ++c) {
                     float* orow = sh.orow[cbase + c];
-                    if (orow == nullptr || hh * 128 + q * 32 + lane >= p.hd) continue;
-                    if (nsplit == 1) orow[hh * 128 + q * 32 + lane] = v[c];
-                    else atomicAdd(orow + hh * 128 + q * 32 + lane, v[c]);
+                    if (orow != nullptr) atomicAdd(orow + hh * 128 + q * 32 + lane, v[c]);
                 }
             }
         }
@@ -1113,8 +1079,6 @@ int attn_chunk_launch(spark_ctx* ctx, const float* q, const void* k1c, const voi
     p.hd = static_cast<int>(hd); p.r = static_cast<int>(r);
     p.window = static_cast<int>(window > 0x7fffffff ? 0x7fffffff : window);
     p.k_attn = static_cast<int>(k_attn > 0x7fffffff ? 0x7fffffff : k_attn);
-    p.tps = p.T;
-    p.nsub = 1;
     p.ncol = static_cast<int>(T * gq);
     p.ncolp = (p.ncol + 15) & ~15;
     p.cap = cap;
@@ -1188,85 +1152,6 @@ int attn_chunk_launch(spark_ctx* ctx, const float* q, const void* k1c, const voi
             return SPARK_ERR_CUDA;
     }
     return SPARK_OK;
-}
-
-// ---- a span of a prompt: many sub-chunks in each launch ---------------------------------------------------------------------
-// The same three kernels (scores, stats, dense) over T consecutive tokens: virtual heads multiply the blocks, so that a span of
-// 1024 tokens fills the GPU where a chunk of 64 leaves each launch with two or three tiles per block and a boundary behind it.
-// Always the dense second stage: with the GPU full its work per column and 128 rows (2.9 us per 64 columns and SM) beats the
-// gather's rows out of L2 up to about ten thousand rows, and grows past that no faster than the scores themselves.
-size_t attn_span_bytes(int64_t T, int64_t n_q, int64_t n_kv, int64_t hd, int64_t r, int64_t rows) {
-    const int64_t gq = n_q / n_kv, tps = kColMax / gq, cols = (T + tps - 1) / tps * n_kv * kColMax;
-    return round_up(static_cast<size_t>(T) * (sizeof(double) + 2 * sizeof(int)), 1024) + 2 * round_up(static_cast<size_t>(cols) * r * 2, 1024) +
-           2 * round_up(static_cast<size_t>(cols) * (hd - r) * 2, 1024) + round_up(static_cast<size_t>(cols) * (((rows + 3) & ~3) + 32) * 4, 1024) +
-           round_up(static_cast<size_t>(cols) * sizeof(float4) + static_cast<size_t>(T) * n_q * 4, 1024);
-}
-
-void attn_span_layout(AttnSpan& a, char* w) {
-    const int64_t gq = a.n_q / a.n_kv, d2 = a.hd - a.r;
-    a.tps = static_cast<int>(kColMax / gq);
-    a.nsub = static_cast<int>((a.T + a.tps - 1) / a.tps);
-    a.colcap = kColMax;
-    const size_t cols = static_cast<size_t>(a.nsub) * a.n_kv * kColMax;
-    a.scap = ((a.rows + 3) & ~static_cast<int64_t>(3)) + 32;
-    a.zt = reinterpret_cast<double*>(w);
-    a.range = reinterpret_cast<int*>(w + a.T * sizeof(double)); w += round_up(static_cast<size_t>(a.T) * (sizeof(double) + 2 * sizeof(int)), 1024);
-    a.qhi = reinterpret_cast<__nv_bfloat16*>(w); w += round_up(cols * a.r * 2, 1024);
-    a.qlo = reinterpret_cast<__nv_bfloat16*>(w); w += round_up(cols * a.r * 2, 1024);
-    a.q2hi = reinterpret_cast<__nv_bfloat16*>(w); w += round_up(cols * d2 * 2, 1024);
-    a.q2lo = reinterpret_cast<__nv_bfloat16*>(w); w += round_up(cols * d2 * 2, 1024);
-    a.S = reinterpret_cast<float*>(w); w += round_up(cols * a.scap * 4, 1024);
-    a.colinfo = reinterpret_cast<float4*>(w);
-    a.zsum = reinterpret_cast<float*>(w + cols * sizeof(float4));
-}
-
-int attn_span_launch(spark_ctx* ctx, const AttnSpan& a, cudaStream_t stream) {
-    if (a.nsub > kMaxSub) return SPARK_ERR_WORKSPACE;
-    const int64_t d2 = a.hd - a.r, vheads = static_cast<int64_t>(a.nsub) * a.n_kv;
-    const size_t smem_dense = static_cast<size_t>(kDSlots) * kDSlotBytes + kDQBytes + 2 * kDWBytes + 1024;
-    const size_t smem_scores = static_cast<size_t>(kChunkStages) * kChunkStageBytes + 1024;
-    if (smem_dense + sizeof(DenseShared) + 64 > static_cast<size_t>(ctx->max_smem_optin) ||
-        smem_scores + sizeof(ChunkShared) + 64 > static_cast<size_t>(ctx->max_smem_optin))
-        return SPARK_ERR_WORKSPACE;
-    ChunkParams p = {};
-    p.T = static_cast<int>(a.T); p.n_q = static_cast<int>(a.n_q); p.n_kv = static_cast<int>(a.n_kv); p.gq = static_cast<int>(a.n_q / a.n_kv);
-    p.hd = static_cast<int>(a.hd); p.r = static_cast<int>(a.r);
-    p.window = static_cast<int>(a.window > 0x7fffffff ? 0x7fffffff : a.window);
-    p.k_attn = static_cast<int>(a.k_attn > 0x7fffffff ? 0x7fffffff : a.k_attn);
-    p.tps = a.tps; p.nsub = a.nsub;
-    p.ncol = p.tps * p.gq;
-    p.ncolp = p.ncol;
-    p.cap = a.cap; p.scap = a.scap;
-    p.o = a.o; p.lsum = a.lsum;
-    p.zt = a.zt; p.range = a.range; p.qhi = a.qhi; p.qlo = a.qlo; p.S = a.S; p.q2hi = a.q2hi; p.q2lo = a.q2lo;
-    p.colinfo = a.colinfo; p.zsum = a.zsum;
-    p.dense = 1;
-    p.hdr = ctx->hdr;
-    CUtensorMap m_k1, m_qhi, m_qlo, m_k2, m_v, m_q2hi, m_q2lo;
-    if (!make_map(&m_k1, a.k1c, a.n_kv * a.cap, a.r, a.r, 128, true) || !make_map(&m_qhi, a.qhi, vheads * kColMax, a.r, a.r, p.ncolp, false) ||
-        !make_map(&m_qlo, a.qlo, vheads * kColMax, a.r, a.r, p.ncolp, false) || !make_map(&m_k2, a.k2c, a.n_kv * a.cap, d2, d2, 128, true) ||
-        !make_map(&m_v, a.vc, a.n_kv * a.cap, a.hd, a.hd, 128, true) || !make_map(&m_q2hi, a.q2hi, vheads * kColMax, d2, d2, kDN, false) ||
-        !make_map(&m_q2lo, a.q2lo, vheads * kColMax, d2, d2, kDN, false))
-        return SPARK_ERR_WORKSPACE;
-    if (cudaFuncSetAttribute(attn_chunk_scores_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem_scores)) != cudaSuccess ||
-        cudaFuncSetAttribute(attn_chunk_dense_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem_dense)) != cudaSuccess)
-        return SPARK_ERR_CUDA;
-    {
-        void* args[] = {&p, &m_k1, &m_qhi, &m_qlo};
-        if (launch_kernel(ctx, reinterpret_cast<const void*>(attn_chunk_scores_kernel), static_cast<unsigned>(ctx->num_sms), kChunkThreads, smem_scores, stream, false, args, true) != cudaSuccess)
-            return SPARK_ERR_CUDA;
-    }
-    {
-        void* args[] = {&p};
-        if (launch_kernel(ctx, reinterpret_cast<const void*>(attn_chunk_stats_kernel), static_cast<unsigned>(a.T * a.n_q), 256, 0, stream, false, args, true) != cudaSuccess)
-            return SPARK_ERR_CUDA;
-    }
-    const int groups = static_cast<int>(vheads) * ((p.ncol + kDN - 1) / kDN);
-    int nsplit = ctx->num_sms / groups;
-    if (nsplit < 1) nsplit = 1;
-    void* args[] = {&p, &m_k2, &m_v, &m_q2hi, &m_q2lo, &nsplit};
-    return launch_kernel(ctx, reinterpret_cast<const void*>(attn_chunk_dense_kernel), static_cast<unsigned>(groups * nsplit), kDThreads, smem_dense, stream, false, args, true) == cudaSuccess
-               ? SPARK_OK : SPARK_ERR_CUDA;
 }
 
 }  // namespace spark

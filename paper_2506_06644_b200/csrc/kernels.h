@@ -68,41 +68,38 @@ int attn_chunk_launch(spark_ctx* ctx, const float* q, const void* k1c, const voi
                       int64_t n_kv, int64_t hd, int64_t r, int64_t cap, const int32_t* ctx_len, const double* zs, int64_t window,
                       int64_t k_attn, float* o, float* lsum, float* theta, int32_t* count, cudaStream_t stream);
 
-// The same for a span of a prompt: T consecutive tokens of one sequence, token t at cache row start + t, queries already split
-// into two bf16 terms per (virtual head, column) -- see attn_chunk.cu.  attn_span_layout places the arrays in `w`
-// (attn_span_bytes of it; rows = cached rows the span's last token sees) and sets the column arithmetic; the caller fills zt,
-// range and the query operands, attn_span_launch leaves the weighted value sums in o and the sums of weights in lsum.
+// Spark attention for a span of a prompt (span_attn.cu): T consecutive tokens of one sequence, token t at cache row start + t,
+// queries already split into two bf16 terms, a row per (virtual head, column).  attn_span_layout places the arrays in `w`
+// (attn_span_bytes of it) and sets the column arithmetic (false: not served); the caller fills zt and the query operands and clears
+// sums, smax, o and lsum; attn_span_launch leaves the weighted value sums in o and the sums of weights in lsum.
 struct AttnSpan {
     const void* k1c;
     const void* k2c;
     const void* vc;
-    int64_t T, n_q, n_kv, hd, r, cap, rows, window, k_attn;
+    int64_t T, n_q, n_kv, hd, r, cap, start, window, k_attn;
     float* o;                // [T][n_q][hd]
     float* lsum;             // [T][n_q]
     int tps, nsub, colcap;   // tokens per sub-chunk, sub-chunks, operand rows per virtual head
-    int64_t scap;
     double* zt;              // [T] Q(1 - k_attn / L_t)
-    int* range;              // [T][2]
+    double* sums;            // [columns][2]
+    unsigned* smax;          // [columns]
     __nv_bfloat16* qhi;      // [nsub * n_kv][colcap][r]
     __nv_bfloat16* qlo;
     __nv_bfloat16* q2hi;     // [nsub * n_kv][colcap][hd - r]
     __nv_bfloat16* q2lo;
-    float* S;
-    float4* colinfo;
-    float* zsum;
 };
-size_t attn_span_bytes(int64_t T, int64_t n_q, int64_t n_kv, int64_t hd, int64_t r, int64_t rows);
-void attn_span_layout(AttnSpan& a, char* w);
+size_t attn_span_bytes(int64_t T, int64_t n_q, int64_t n_kv, int64_t hd);
+bool attn_span_layout(AttnSpan& a, char* w);
 int attn_span_launch(spark_ctx* ctx, const AttnSpan& a, cudaStream_t stream);
 
 // A span of a prompt (T consecutive tokens of one sequence, cached rows start .. start + T - 1) through one layer (span.cu), in
 // the workspace of ctx.  span_tokens: the most tokens the workspace has room for with these layers, or 0 when a layer's shape,
 // flags or pointers are not served.
 int64_t span_tokens(const spark_ctx* ctx, const spark_layer_weights* w, const spark_layer_cfg* cfg, const spark_kv_cache* cache, int64_t n_layers,
-                    const float* h, int64_t n_tokens, int64_t start);
+                    const float* h, int64_t n_tokens);
 int span_layer_launch(spark_ctx* ctx, const spark_layer_weights* w, const spark_layer_cfg* cfg, const spark_kv_cache* cache, float* h, int64_t T,
                       int64_t start, cudaStream_t stream);
-size_t span_workspace_bytes(int64_t max_dff, int64_t max_cap, int64_t n_q, int64_t hd, int64_t max_d);
+size_t span_workspace_bytes(int64_t max_dff, int64_t n_q, int64_t hd, int64_t max_d);
 
 // One token through n_layers decoder layers in one launch of the fused persistent kernel (layer1.cu); the layers' configurations
 // are equal but for the attention window.  SPARK_ERR_WORKSPACE = shape, flags or sizes not served.

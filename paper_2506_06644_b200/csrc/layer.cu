@@ -802,7 +802,7 @@ extern "C" int spark_prefill(spark_ctx* ctx, const spark_layer_weights* w, const
     if (!on_device(ctx)) return SPARK_ERR_INVALID_ARG;
     cudaStream_t st = static_cast<cudaStream_t>(stream);
     // as many tokens at a time as the workspace holds, when the layers allow it (span.cu)
-    if (const int64_t span = span_tokens(ctx, w, cfg, cache, n_layers, h, n_tokens, start)) return prefill_spans(ctx, w, cfg, cache, n_layers, h, n_tokens, start, span, st);
+    if (const int64_t span = span_tokens(ctx, w, cfg, cache, n_layers, h, n_tokens)) return prefill_spans(ctx, w, cfg, cache, n_layers, h, n_tokens, start, span, st);
     for (int64_t c0 = 0; c0 < n_tokens; c0 += chunk) {
         const int64_t T = n_tokens - c0 < chunk ? n_tokens - c0 : chunk;
         int n = static_cast<int>(T), first = static_cast<int>(start + c0 + 1);
@@ -848,7 +848,7 @@ extern "C" int spark_prefill_pipelined(spark_ctx* const* ctxs, float* const* scr
     cudaStream_t st[kMaxInflight];
     for (int i = 0; i < n; ++i) st[i] = static_cast<cudaStream_t>(streams[i]);
     // spans fill the GPU by themselves: they run on the first context and stream, where the call forks from and joins
-    if (const int64_t span = span_tokens(ctxs[0], w, cfg, cache, n_layers, h, n_tokens, start))
+    if (const int64_t span = span_tokens(ctxs[0], w, cfg, cache, n_layers, h, n_tokens))
         return prefill_spans(ctxs[0], w, cfg, cache, n_layers, h, n_tokens, start, span, st[0]);
     // done[s][l]: layer l of the newest chunk on stream s has finished; fork and join around the call
     const size_t n_ev = static_cast<size_t>(n) * static_cast<size_t>(n_layers) + 1 + static_cast<size_t>(n);

@@ -7,8 +7,8 @@
 // tiles fastest so that a weight tile comes from HBM once.  Every product of more than 2304 columns is cut into segments that
 // alternate between two tensor-memory accumulators; the epilogue warps add the segments in fp32, which keeps the accumulator's
 // truncation at 144 steps and hides the epilogue of a tile under the next one.  Kernels per layer and span:
-//   prep (norm1) -> QKV -> rope (queries into operand form, cache append, quantiles) -> attention (scores, stats, dense; see
-//   attn_chunk.cu) -> prep (softmax division) -> Wo + h -> prep (norm2) -> K1 scores -> theta -> K2, whose epilogue forms
+//   prep (norm1) -> QKV -> rope (queries into operand form, cache append, quantiles) -> attention (two kernels, span_attn.cu)
+//   -> prep (softmax division) -> Wo + h -> prep (norm2) -> K1 scores -> theta -> K2, whose epilogue forms
 //   u = [s > theta] GELU(s - theta) t in two bf16 terms -> V + h2
 // 4000 tokens through eight layers of the 2B shape: 45.9 ms in 64-token calls.
 #include <cmath>
@@ -162,6 +162,7 @@ span_gemm_kernel(const SpanGemm p, const __grid_constant__ CUtensorMap map_w, co
         for (int tile = blockIdx.x; tile < p.tiles && ok; tile += gridDim.x) {
             const int m = tile / p.tiles_t, tt = tile - m * p.tiles_t;
             const int row = m * 128 + q * 32 + lane, t0 = tt * kSpanTile + half * 64;
+            const int64_t at = static_cast<int64_t>(t0) * p.rows + row;
             float acc[64];
             for (int g = 0; g < p.nseg; ++g, ++seg) {
                 const int b = seg & 1;
@@ -182,7 +183,6 @@ span_gemm_kernel(const SpanGemm p, const __grid_constant__ CUtensorMap map_w, co
             }
             if (!ok) break;
             if (row >= p.rows) continue;
-            const int64_t at = static_cast<int64_t>(t0) * p.rows + row;
             if constexpr (U) {
                 __nv_bfloat16* uh = p.u + at;
                 __nv_bfloat16* ul = uh + static_cast<int64_t>(p.lo_row) * p.rows;
@@ -354,22 +354,31 @@ struct SpanRope {
     int64_t cap;
     float q_scale;
     double* zt;
-    int* range;
+    double* sums;            // cleared for the attention, like smax, o and lsum
+    unsigned* smax;
+    float* o;                // [T][n_q][hd]
+    float* lsum;             // [T][n_q]
     __nv_bfloat16* qhi;
     __nv_bfloat16* qlo;
     __nv_bfloat16* q2hi;
     __nv_bfloat16* q2lo;
     double inv_freq[2][64];
 };
-__global__ void __launch_bounds__(128) span_rope_kernel(const __grid_constant__ SpanRope p) {
-    const int t = blockIdx.x, pr = threadIdx.x, pos = p.start + t, hr = p.r / 2;
+__global__ void __launch_bounds__(256) span_rope_kernel(const __grid_constant__ SpanRope p) {
+    // two groups of 128 threads take every other head
+    const int t = blockIdx.x, pr = threadIdx.x & 127, grp = threadIdx.x >> 7, pos = p.start + t, hr = p.r / 2;
     const int sub = t / p.tps, col0 = (t - sub * p.tps) * p.gq;
     dep_wait();
     dep_trigger();
-    if (pr == 127) {         // the rows the token sees and the threshold quantile over them
+    for (int i = threadIdx.x; i < p.n_q * p.hd / 4; i += 256) reinterpret_cast<float4*>(p.o + static_cast<int64_t>(t) * p.n_q * p.hd)[i] = make_float4(0.f, 0.f, 0.f, 0.f);
+    for (int h = threadIdx.x; h < p.n_q; h += 256) {
+        const int64_t vcol = static_cast<int64_t>(sub * p.n_kv + h / p.gq) * p.colcap + col0 + h % p.gq;
+        p.sums[2 * vcol] = p.sums[2 * vcol + 1] = 0.0;
+        p.smax[vcol] = 0u;
+        p.lsum[static_cast<int64_t>(t) * p.n_q + h] = 0.f;
+    }
+    if (threadIdx.x == 255) {         // the threshold quantile over the rows the token sees
         const int n = pos + 1, L = (p.window > 0 && p.window < n) ? p.window : n;
-        p.range[2 * t] = n - L;
-        p.range[2 * t + 1] = n;
         p.zt[t] = p.k_attn >= L ? 0.0 : -normcdfinv(static_cast<double>(p.k_attn) / static_cast<double>(L));
     }
     if (pr >= p.hd / 2) return;
@@ -384,7 +393,7 @@ __global__ void __launch_bounds__(128) span_rope_kernel(const __grid_constant__ 
     const float* row = p.qkv + static_cast<int64_t>(t) * (p.n_q + 2 * p.n_kv) * p.hd;
     __nv_bfloat16* oh = second ? p.q2hi : p.qhi;
     __nv_bfloat16* ol = second ? p.q2lo : p.qlo;
-    for (int h = 0; h < p.n_q; ++h) {
+    for (int h = grp; h < p.n_q; h += 2) {
         const float a = row[h * p.hd + ia], b = row[h * p.hd + ib];
         const float ra = (a * cs - b * sn) * p.q_scale, rb = (a * sn + b * cs) * p.q_scale;
         const int g = h / p.gq;
@@ -396,7 +405,7 @@ __global__ void __launch_bounds__(128) span_rope_kernel(const __grid_constant__ 
         ol[at + m / 2] = __float2bfloat16_rn(rb - __bfloat162float(hb));
     }
     __nv_bfloat16* kc = second ? p.k2c : p.k1c;
-    for (int g = 0; g < p.n_kv; ++g) {
+    for (int g = grp; g < p.n_kv; g += 2) {
         const float* src = row + static_cast<int64_t>(p.n_q + g) * p.hd;
         const float a = src[ia], b = src[ib];
         __nv_bfloat16* dst = kc + (g * p.cap + pos) * m + pi;
@@ -413,7 +422,7 @@ struct SpanLayout {
     int64_t Tp;
     size_t xs, qkv, ao, lsum, h2, theta, shared, S, u, bytes;
 };
-SpanLayout span_layout(int64_t T, int64_t d, int64_t d_ff, int64_t n_q, int64_t n_kv, int64_t hd, int64_t r, int64_t rows) {
+SpanLayout span_layout(int64_t T, int64_t d, int64_t d_ff, int64_t n_q, int64_t n_kv, int64_t hd) {
     SpanLayout l;
     l.Tp = (T + kSpanTile - 1) / kSpanTile * kSpanTile;
     const size_t Tp = static_cast<size_t>(l.Tp), nqo = static_cast<size_t>(n_q * hd), nqkv = static_cast<size_t>((n_q + 2 * n_kv) * hd);
@@ -430,7 +439,7 @@ SpanLayout span_layout(int64_t T, int64_t d, int64_t d_ff, int64_t n_q, int64_t 
     l.h2 = take(Tp * static_cast<size_t>(d) * 4);
     l.theta = take(Tp * 4);
     l.shared = at;
-    const size_t attn = attn_span_bytes(l.Tp, n_q, n_kv, hd, r, rows);
+    const size_t attn = attn_span_bytes(l.Tp, n_q, n_kv, hd);
     l.S = take(Tp * static_cast<size_t>(d_ff) * 4);
     l.u = take(2 * Tp * static_cast<size_t>(d_ff) * 2);
     l.bytes = at > l.shared + attn ? at : l.shared + attn;
@@ -463,19 +472,15 @@ int span_gemm(spark_ctx* ctx, SpanGemm p, const void* W, int64_t K, const __nv_b
 
 namespace spark {
 
-size_t span_workspace_bytes(int64_t max_dff, int64_t max_cap, int64_t n_q, int64_t hd, int64_t max_d) {
-    if (max_dff < 8 || max_d < 16 || max_cap < 1) return 0;
-    // the tokens whose score matrix (n_q columns of max_cap rows each) takes up to 192 MB, but at least one tile of them
-    int64_t T = (192ll << 20) / (n_q * (max_cap + 35) * 4) / kSpanTile * kSpanTile;
-    T = T < kSpanTile ? kSpanTile : (T > kSpanMax ? kSpanMax : T);
-    return kAttnCellBytes + span_layout(T, max_d, max_dff, n_q, n_q, hd, hd / 2, max_cap).bytes;
+size_t span_workspace_bytes(int64_t max_dff, int64_t n_q, int64_t hd, int64_t max_d) {
+    if (max_dff < 8 || max_d < 16) return 0;
+    return kAttnCellBytes + span_layout(kSpanMax, max_d, max_dff, n_q, n_q, hd).bytes;
 }
 
 int64_t span_tokens(const spark_ctx* ctx, const spark_layer_weights* w, const spark_layer_cfg* cfg, const spark_kv_cache* cache, int64_t n_layers,
-                    const float* h, int64_t n_tokens, int64_t start) {
+                    const float* h, int64_t n_tokens) {
     if (n_tokens <= 64 || ctx->chunk_dense == 0 || ctx->scratch == nullptr || (reinterpret_cast<uintptr_t>(h) & 15u) != 0) return 0;
     int64_t T = n_tokens < kSpanMax ? n_tokens : kSpanMax;
-    const int64_t rows = start + n_tokens;
     for (int64_t l = 0; l < n_layers; ++l) {
         const spark_layer_cfg& c = cfg[l];
         if ((c.flags & ~(SPARK_GELU_ERF | SPARK_SHARED_CACHE)) != 0) return 0;
@@ -490,7 +495,7 @@ int64_t span_tokens(const spark_ctx* ctx, const spark_layer_weights* w, const sp
         const void* need[] = {w[l].norm1, w[l].norm2, w[l].Wqkv, w[l].Wo, w[l].K1t, w[l].K2t, w[l].Vt, cache[l].k1c, cache[l].k2c, cache[l].vc};
         for (const void* ptr : need)
             if (ptr == nullptr || (reinterpret_cast<uintptr_t>(ptr) & 15u) != 0) return 0;
-        while (T > 64 && kAttnCellBytes + span_layout(T, c.d, c.d_ff, c.n_q, c.n_kv, c.hd, c.r_attn, rows).bytes > ctx->scratch_bytes)
+        while (T > 64 && kAttnCellBytes + span_layout(T, c.d, c.d_ff, c.n_q, c.n_kv, c.hd).bytes > ctx->scratch_bytes)
             T = (T - 1) / kSpanTile * kSpanTile;
     }
     if (T <= 64) return 0;
@@ -502,7 +507,7 @@ int64_t span_tokens(const spark_ctx* ctx, const spark_layer_weights* w, const sp
 int span_layer_launch(spark_ctx* ctx, const spark_layer_weights* w, const spark_layer_cfg* cfg, const spark_kv_cache* cache, float* h, int64_t T,
                       int64_t start, cudaStream_t stream) {
     const int64_t d = cfg->d, d_ff = cfg->d_ff, n_q = cfg->n_q, n_kv = cfg->n_kv, hd = cfg->hd, nqo = n_q * hd, nqkv = (n_q + 2 * n_kv) * hd;
-    const SpanLayout l = span_layout(T, d, d_ff, n_q, n_kv, hd, cfg->r_attn, start + T);
+    const SpanLayout l = span_layout(T, d, d_ff, n_q, n_kv, hd);
     char* base = ctx->scratch + kAttnCellBytes;
     __nv_bfloat16* xs = reinterpret_cast<__nv_bfloat16*>(base + l.xs);
     float* qkv = reinterpret_cast<float*>(base + l.qkv);
@@ -530,10 +535,10 @@ int span_layer_launch(spark_ctx* ctx, const spark_layer_weights* w, const spark_
 
     AttnSpan a;
     a.k1c = cache->k1c; a.k2c = cache->k2c; a.vc = cache->vc;
-    a.T = T; a.n_q = n_q; a.n_kv = n_kv; a.hd = hd; a.r = cfg->r_attn; a.cap = cfg->cap; a.rows = start + T;
+    a.T = T; a.n_q = n_q; a.n_kv = n_kv; a.hd = hd; a.r = cfg->r_attn; a.cap = cfg->cap; a.start = start;
     a.window = cfg->window; a.k_attn = cfg->k_attn;
     a.o = ao; a.lsum = lsum;
-    attn_span_layout(a, base + l.shared);
+    if (!attn_span_layout(a, base + l.shared)) return SPARK_ERR_UNSUPPORTED;
     {
         SpanRope p;
         p.qkv = qkv;
@@ -544,14 +549,14 @@ int span_layer_launch(spark_ctx* ctx, const spark_layer_weights* w, const spark_
         p.k_attn = static_cast<int>(cfg->k_attn > 0x7fffffff ? 0x7fffffff : cfg->k_attn);
         p.cap = cfg->cap;
         p.q_scale = 1.0f / std::sqrt(static_cast<float>(hd));
-        p.zt = a.zt; p.range = a.range; p.qhi = a.qhi; p.qlo = a.qlo; p.q2hi = a.q2hi; p.q2lo = a.q2lo;
+        p.zt = a.zt; p.sums = a.sums; p.smax = a.smax; p.o = ao; p.lsum = lsum; p.qhi = a.qhi; p.qlo = a.qlo; p.q2hi = a.q2hi; p.q2lo = a.q2lo;
         for (int part = 0; part < 2; ++part) {
             const int64_t m = part == 0 ? cfg->r_attn : hd - cfg->r_attn;
             for (int64_t i = 0; i < m / 2; ++i)
                 p.inv_freq[part][i] = std::pow(static_cast<double>(cfg->rope_base), -2.0 * static_cast<double>(i) / static_cast<double>(m));
         }
         void* args[] = {&p};
-        if (launch_kernel(ctx, reinterpret_cast<const void*>(span_rope_kernel), static_cast<unsigned>(T), 128, 0, stream, false, args, true) != cudaSuccess) return SPARK_ERR_CUDA;
+        if (launch_kernel(ctx, reinterpret_cast<const void*>(span_rope_kernel), static_cast<unsigned>(T), 256, 0, stream, false, args, true) != cudaSuccess) return SPARK_ERR_CUDA;
     }
     rc = attn_span_launch(ctx, a, stream);
     if (rc == SPARK_OK) rc = prep(ao, nullptr, lsum, nqo, hd);

@@ -74,7 +74,7 @@ size_t spark_workspace_bytes(int64_t max_batch, int64_t max_dff, int64_t max_cap
                      round_up(static_cast<size_t>(n_q) * 128 * (static_cast<size_t>(max_cap) + 32) * 4, 1024) +
                      round_up(static_cast<size_t>(n_q) * (128 * 16 + 64 * 4), 1024) + 1024;                    // column facts of the dense stage
     // prefill: a span of a prompt through a layer (contexts made for chunks of 32 tokens and more)
-    const size_t need_span = max_batch >= 32 ? span_workspace_bytes(max_dff, max_cap, n_q, hd, max_d) : 0;
+    const size_t need_span = max_batch >= 32 ? span_workspace_bytes(max_dff, n_q, hd, max_d) : 0;
     size_t most = need > need_ffn ? need : need_ffn;
     if (need_chunk > most) most = need_chunk;
     if (need_span > most) most = need_span;
