@@ -52,6 +52,14 @@ struct SpanShared {
     int abort_flag;
 };
 
+// The tanh form of GELU as a x sigmoid(2 sqrt(2/pi) (a + 0.044715 a^3)): the same function with one exponential and one division.
+__device__ __forceinline__ float gelu_logistic(float a) {
+    const float y = a * fmaf(0.1029432397f, a * a, 2.302208198f);      // 2 sqrt(2/pi) log2(e) (1, 0.044715)
+    float e;
+    asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(e) : "f"(-y));
+    return __fdividef(a, 1.f + e);
+}
+
 // MN: the matrix is stored [K][rows] (V); U: the epilogue forms the activations.
 template <bool MN, bool U>
 __global__ void __launch_bounds__(kSpanThreads, 1)
@@ -163,6 +171,47 @@ span_gemm_kernel(const SpanGemm p, const __grid_constant__ CUtensorMap map_w, co
             const int m = tile / p.tiles_t, tt = tile - m * p.tiles_t;
             const int row = m * 128 + q * 32 + lane, t0 = tt * kSpanTile + half * 64;
             const int64_t at = static_cast<int64_t>(t0) * p.rows + row;
+            if constexpr (U) {
+                // one segment; sixteen tokens at a time: scores in, activation, two bf16 terms out
+                const int b = seg & 1;
+                ok = __all_sync(kFull, mbar_wait(smem_addr(&sh.acc_full[b]), (seg >> 1) & 1, abort_flag));
+                if (!ok) break;
+                ++seg;
+                tc_fence_after();
+                const uint32_t taddr = tmem + static_cast<uint32_t>(b * 256 + half * 64) + (static_cast<uint32_t>(q * 32) << 16);
+                const bool odd = lane & 1;
+                // even lanes store this pair of rows for the even tokens, odd lanes for the odd ones
+                __nv_bfloat16* uh = p.u + at + (odd ? static_cast<int64_t>(p.rows) - 1 : 0);
+                const int64_t lo = static_cast<int64_t>(p.lo_row) * p.rows;
+#pragma unroll 1
+                for (int j = 0; j < 4; ++j) {
+                    float sv[16], v[16];
+#pragma unroll
+                    for (int i = 0; i < 16; ++i)
+                        sv[i] = row < p.rows && t0 + 16 * j + i < p.T ? __ldcg(p.S + at + static_cast<int64_t>(16 * j + i) * p.rows) : -INFINITY;
+                    tmem_ld16_sum(taddr + 16 * j, taddr + kSpanTile + 16 * j, v);
+#pragma unroll
+                    for (int i = 0; i < 16; ++i) {
+                        const float th = __ldg(p.theta + min(t0 + 16 * j + i, p.T - 1));
+                        const float a = p.identity ? sv[i] : sv[i] - th;
+                        v[i] = sv[i] > th ? (p.erf_form ? gelu_erf(a) : gelu_logistic(a)) * v[i] : 0.f;
+                    }
+#pragma unroll
+                    for (int i = 0; i < 16; i += 2) {
+                        const float mine = odd ? v[i + 1] : v[i], other = __shfl_xor_sync(kFull, odd ? v[i] : v[i + 1], 1);
+                        unsigned hi, l;
+                        split_pair(odd ? other : mine, odd ? mine : other, hi, l);
+                        if (row < p.rows && t0 + 16 * j + i + (odd ? 1 : 0) < p.T) {
+                            __nv_bfloat16* dst = uh + static_cast<int64_t>(16 * j + i) * p.rows;
+                            *reinterpret_cast<unsigned*>(dst) = hi;
+                            *reinterpret_cast<unsigned*>(dst + lo) = l;
+                        }
+                    }
+                }
+                tc_fence_before();
+                __syncwarp();
+                if (lane == 0) asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_addr(&sh.acc_empty[b])) : "memory");
+            } else {
             float acc[64];
             for (int g = 0; g < p.nseg; ++g, ++seg) {
                 const int b = seg & 1;
@@ -183,32 +232,6 @@ span_gemm_kernel(const SpanGemm p, const __grid_constant__ CUtensorMap map_w, co
             }
             if (!ok) break;
             if (row >= p.rows) continue;
-            if constexpr (U) {
-                __nv_bfloat16* uh = p.u + at;
-                __nv_bfloat16* ul = uh + static_cast<int64_t>(p.lo_row) * p.rows;
-#pragma unroll
-                for (int j = 0; j < 4; ++j) {
-                    float sv[16], th[16];
-#pragma unroll
-                    for (int i = 0; i < 16; ++i) {
-                        const bool in = t0 + 16 * j + i < p.T;
-                        sv[i] = in ? __ldcg(p.S + at + static_cast<int64_t>(16 * j + i) * p.rows) : 0.f;
-                        th[i] = in ? __ldcg(p.theta + t0 + 16 * j + i) : INFINITY;
-                    }
-#pragma unroll
-                    for (int i = 0; i < 16; ++i) {
-                        if (t0 + 16 * j + i >= p.T) break;
-                        float u = 0.f;
-                        if (sv[i] > th[i]) {
-                            const float a = p.identity ? sv[i] : sv[i] - th[i];
-                            u = (p.erf_form ? gelu_erf(a) : gelu_tanh(a)) * acc[16 * j + i];
-                        }
-                        const __nv_bfloat16 hi = __float2bfloat16_rn(u);
-                        uh[static_cast<int64_t>(16 * j + i) * p.rows] = hi;
-                        ul[static_cast<int64_t>(16 * j + i) * p.rows] = __float2bfloat16_rn(u - __bfloat162float(hi));
-                    }
-                }
-            } else {
 #pragma unroll
                 for (int j = 0; j < 4; ++j) {
                     float av[16];
@@ -451,7 +474,7 @@ template <bool MN, bool U>
 int span_gemm(spark_ctx* ctx, SpanGemm p, const void* W, int64_t K, const __nv_bfloat16* X, int64_t ldx, int64_t Tp, cudaStream_t stream) {
     const int tiles_m = (p.rows + 127) / 128;
     p.call = static_cast<int>((K + kChunk - 1) / kChunk);
-    p.nseg = (p.call + kSpanSeg - 1) / kSpanSeg;
+    p.nseg = U ? 1 : (p.call + kSpanSeg - 1) / kSpanSeg;
     p.tiles_t = static_cast<int>((p.T + kSpanTile - 1) / kSpanTile);
     p.tiles = tiles_m * p.tiles_t;
     p.lo_row = static_cast<int>(Tp);
