@@ -10,7 +10,7 @@
 //   prep (norm1) -> QKV -> rope (queries into operand form, cache append, quantiles) -> attention (two kernels, span_attn.cu)
 //   -> prep (softmax division) -> Wo + h -> prep (norm2) -> K1 scores -> theta -> K2, whose epilogue forms
 //   u = [s > theta] GELU(s - theta) t in two bf16 terms -> V + h2
-// 4000 tokens through eight layers of the 2B shape: 45.9 ms in 64-token calls.
+// 4000 tokens through eight layers of the 2B shape: 45.9 ms in 64-token calls, 9.5 ms this way.
 #include <cmath>
 
 #include "ffn_params.h"
@@ -32,8 +32,9 @@ constexpr int kSpanThreads = 64 + 8 * 32;      // warp 0: TMA, warp 1: MMA + ten
 
 struct SpanGemm {
     int rows, T, call;
-    int tiles_t, tiles;      // token tiles; all tiles
-    int nseg;                // segments of a tile
+    int tiles_t, tiles;      // token tiles; all work items: tiles, or pieces of tiles
+    int split;               // pieces of a tile's K range, added into y with reductions (1: none)
+    int nseg;                // segments of an item
     int lo_row;              // rows of X's second term start here
     const float* add;        // nullable [T][rows]
     float* y;                // [T][rows]
@@ -87,6 +88,13 @@ span_gemm_kernel(const SpanGemm p, const __grid_constant__ CUtensorMap map_w, co
     const uint32_t base = (smem_addr(tc_raw) + 1023u) & ~1023u;
     const uint32_t tmem = sh.tmem;
     volatile int* abort_flag = &sh.abort_flag;
+    struct Item {
+        int m, tt, c0, c1;       // row tile, token tile, K chunks
+    };
+    auto item = [&](int i) -> Item {
+        const int tile = i / p.split, k = i - tile * p.split, m = tile / p.tiles_t;
+        return Item{m, tile - m * p.tiles_t, k * p.call / p.split, (k + 1) * p.call / p.split};
+    };
     dep_trigger();           // the kernel behind does not touch what it shares with this one before its wait
 
     if (warp == 0) {
@@ -110,19 +118,19 @@ span_gemm_kernel(const SpanGemm p, const __grid_constant__ CUtensorMap map_w, co
             };
             // the first stages of weights do not depend on the kernel ahead
             int pre = 0;
-            const int m0 = blockIdx.x / p.tiles_t, tt0 = blockIdx.x - m0 * p.tiles_t;
+            const Item first = item(blockIdx.x);
             if (static_cast<int>(blockIdx.x) < p.tiles)
-                for (; pre < min(p.call, kSpanStages); ++pre) load_w(pre, m0, pre);
+                for (; pre < min(first.c1 - first.c0, kSpanStages); ++pre) load_w(pre, first.m, first.c0 + pre);
             dep_wait();
-            for (int i = 0; i < pre; ++i) load_x(i, tt0, i);
+            for (int i = 0; i < pre; ++i) load_x(i, first.tt, first.c0 + i);
             bool ok = true;
             for (int tile = blockIdx.x; tile < p.tiles && ok; tile += gridDim.x) {
-                const int m = tile / p.tiles_t, tt = tile - m * p.tiles_t;
-                for (int c = 0; c < p.call; ++c, ++it) {
+                const Item w = item(tile);
+                for (int c = w.c0; c < w.c1; ++c, ++it) {
                     if (it >= pre) {
                         if (it >= kSpanStages && !mbar_wait(smem_addr(&sh.empty[s]), parity, abort_flag)) { ok = false; break; }
-                        load_w(s, m, c);
-                        load_x(s, tt, c);
+                        load_w(s, w.m, c);
+                        load_x(s, w.tt, c);
                     }
                     if (++s == kSpanStages) { s = 0; parity ^= 1u; }
                 }
@@ -141,8 +149,9 @@ span_gemm_kernel(const SpanGemm p, const __grid_constant__ CUtensorMap map_w, co
         uint32_t parity = 0u;
         bool ok = true;
         for (int tile = blockIdx.x; tile < p.tiles && ok; tile += gridDim.x) {
+            const Item w = item(tile);
             for (int g = 0; g < p.nseg && ok; ++g, ++seg) {
-                const int c0 = g * p.call / p.nseg, c1 = (g + 1) * p.call / p.nseg, b = seg & 1;
+                const int c0 = w.c0 + g * (w.c1 - w.c0) / p.nseg, c1 = w.c0 + (g + 1) * (w.c1 - w.c0) / p.nseg, b = seg & 1;
                 if (seg >= 2) ok = __all_sync(kFull, mbar_wait(smem_addr(&sh.acc_empty[b]), ((seg >> 1) & 1) ^ 1, abort_flag));
                 const uint32_t acc = tmem + static_cast<uint32_t>(b) * 256u;
                 tc_fence_after();
@@ -168,11 +177,18 @@ span_gemm_kernel(const SpanGemm p, const __grid_constant__ CUtensorMap map_w, co
         int seg = 0;
         bool ok = true;
         for (int tile = blockIdx.x; tile < p.tiles && ok; tile += gridDim.x) {
-            const int m = tile / p.tiles_t, tt = tile - m * p.tiles_t;
-            const int row = m * 128 + q * 32 + lane, t0 = tt * kSpanTile + half * 64;
+            const Item w = item(tile);
+            const int row = w.m * 128 + q * 32 + lane, t0 = w.tt * kSpanTile + half * 64;
             const int64_t at = static_cast<int64_t>(t0) * p.rows + row;
             if constexpr (U) {
-                // one segment; sixteen tokens at a time: scores in, activation, two bf16 terms out
+                // one segment; sixteen tokens at a time: scores in (one group ahead), activation, two bf16 terms out
+                float next[16];
+                auto request = [&](int j) {
+#pragma unroll
+                    for (int i = 0; i < 16; ++i)
+                        next[i] = row < p.rows && t0 + 16 * j + i < p.T ? __ldcg(p.S + at + static_cast<int64_t>(16 * j + i) * p.rows) : -INFINITY;
+                };
+                request(0);
                 const int b = seg & 1;
                 ok = __all_sync(kFull, mbar_wait(smem_addr(&sh.acc_full[b]), (seg >> 1) & 1, abort_flag));
                 if (!ok) break;
@@ -187,8 +203,8 @@ span_gemm_kernel(const SpanGemm p, const __grid_constant__ CUtensorMap map_w, co
                 for (int j = 0; j < 4; ++j) {
                     float sv[16], v[16];
 #pragma unroll
-                    for (int i = 0; i < 16; ++i)
-                        sv[i] = row < p.rows && t0 + 16 * j + i < p.T ? __ldcg(p.S + at + static_cast<int64_t>(16 * j + i) * p.rows) : -INFINITY;
+                    for (int i = 0; i < 16; ++i) sv[i] = next[i];
+                    if (j < 3) request(j + 1);
                     tmem_ld16_sum(taddr + 16 * j, taddr + kSpanTile + 16 * j, v);
 #pragma unroll
                     for (int i = 0; i < 16; ++i) {
@@ -212,26 +228,32 @@ span_gemm_kernel(const SpanGemm p, const __grid_constant__ CUtensorMap map_w, co
                 __syncwarp();
                 if (lane == 0) asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_addr(&sh.acc_empty[b])) : "memory");
             } else {
-            float acc[64];
-            for (int g = 0; g < p.nseg; ++g, ++seg) {
-                const int b = seg & 1;
-                ok = __all_sync(kFull, mbar_wait(smem_addr(&sh.acc_full[b]), (seg >> 1) & 1, abort_flag));
-                if (!ok) break;
-                tc_fence_after();
-                const uint32_t taddr = tmem + static_cast<uint32_t>(b * 256 + half * 64) + (static_cast<uint32_t>(q * 32) << 16);
+                float acc[64];
+                for (int g = 0; g < p.nseg; ++g, ++seg) {
+                    const int b = seg & 1;
+                    ok = __all_sync(kFull, mbar_wait(smem_addr(&sh.acc_full[b]), (seg >> 1) & 1, abort_flag));
+                    if (!ok) break;
+                    tc_fence_after();
+                    const uint32_t taddr = tmem + static_cast<uint32_t>(b * 256 + half * 64) + (static_cast<uint32_t>(q * 32) << 16);
 #pragma unroll
-                for (int j = 0; j < 4; ++j) {
-                    float v[16];
-                    tmem_ld16_sum(taddr + 16 * j, taddr + kSpanTile + 16 * j, v);
+                    for (int j = 0; j < 4; ++j) {
+                        float v[16];
+                        tmem_ld16_sum(taddr + 16 * j, taddr + kSpanTile + 16 * j, v);
 #pragma unroll
-                    for (int i = 0; i < 16; ++i) acc[16 * j + i] = g == 0 ? v[i] : acc[16 * j + i] + v[i];
+                        for (int i = 0; i < 16; ++i) acc[16 * j + i] = g == 0 ? v[i] : acc[16 * j + i] + v[i];
+                    }
+                    tc_fence_before();
+                    __syncwarp();
+                    if (lane == 0) asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_addr(&sh.acc_empty[b])) : "memory");
                 }
-                tc_fence_before();
-                __syncwarp();
-                if (lane == 0) asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_addr(&sh.acc_empty[b])) : "memory");
-            }
-            if (!ok) break;
-            if (row >= p.rows) continue;
+                if (!ok) break;
+                if (row >= p.rows) continue;
+                if (p.split > 1) {           // y holds the addend already
+#pragma unroll
+                    for (int i = 0; i < 64; ++i)
+                        if (t0 + i < p.T) atomicAdd(p.y + at + static_cast<int64_t>(i) * p.rows, acc[i]);
+                    continue;
+                }
 #pragma unroll
                 for (int j = 0; j < 4; ++j) {
                     float av[16];
@@ -262,6 +284,7 @@ struct SpanPrep {
     const float* div;        // nullable [T][n / group]
     int n, group, lo_row;
     __nv_bfloat16* xs;       // [2 * Tp][n]
+    float* copy;             // nullable: x goes here as well (what a product in pieces adds into)
 };
 __global__ void __launch_bounds__(256) span_prep_kernel(const SpanPrep p) {
     __shared__ float red[8];
@@ -281,6 +304,13 @@ __global__ void __launch_bounds__(256) span_prep_kernel(const SpanPrep p) {
     float4 keep[kKeep];
 #pragma unroll
     for (int u = 0; u < kKeep; ++u) keep[u] = tid + 256 * u < n4 ? load(tid + 256 * u) : make_float4(0.f, 0.f, 0.f, 0.f);
+    if (p.copy != nullptr) {
+        float4* dst = reinterpret_cast<float4*>(p.copy + static_cast<int64_t>(t) * p.n);
+#pragma unroll
+        for (int u = 0; u < kKeep; ++u)
+            if (tid + 256 * u < n4) dst[tid + 256 * u] = keep[u];
+        for (int i = tid + 256 * kKeep; i < n4; i += 256) dst[i] = xr[i];
+    }
     float sc = 1.f;
     if (p.norm_w != nullptr) {
         float ss = 0.f;
@@ -416,26 +446,48 @@ __global__ void __launch_bounds__(256) span_rope_kernel(const __grid_constant__ 
     const float* row = p.qkv + static_cast<int64_t>(t) * (p.n_q + 2 * p.n_kv) * p.hd;
     __nv_bfloat16* oh = second ? p.q2hi : p.qhi;
     __nv_bfloat16* ol = second ? p.q2lo : p.qlo;
-    for (int h = grp; h < p.n_q; h += 2) {
-        const float a = row[h * p.hd + ia], b = row[h * p.hd + ib];
-        const float ra = (a * cs - b * sn) * p.q_scale, rb = (a * sn + b * cs) * p.q_scale;
-        const int g = h / p.gq;
-        const int64_t at = (static_cast<int64_t>(sub * p.n_kv + g) * p.colcap + col0 + h - g * p.gq) * m + pi;
-        const __nv_bfloat16 ha = __float2bfloat16_rn(ra), hb = __float2bfloat16_rn(rb);
-        oh[at] = ha;
-        oh[at + m / 2] = hb;
-        ol[at] = __float2bfloat16_rn(ra - __bfloat162float(ha));
-        ol[at + m / 2] = __float2bfloat16_rn(rb - __bfloat162float(hb));
+    // four heads at a time, their loads in flight together
+    for (int h0 = grp; h0 < p.n_q; h0 += 8) {
+        float a[4], b[4];
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+            const int h = min(h0 + 2 * u, p.n_q - 1);
+            a[u] = __ldg(row + h * p.hd + ia);
+            b[u] = __ldg(row + h * p.hd + ib);
+        }
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+            const int h = h0 + 2 * u, g = h / p.gq;
+            if (h >= p.n_q) break;
+            const float ra = (a[u] * cs - b[u] * sn) * p.q_scale, rb = (a[u] * sn + b[u] * cs) * p.q_scale;
+            const int64_t at = (static_cast<int64_t>(sub * p.n_kv + g) * p.colcap + col0 + h - g * p.gq) * m + pi;
+            const __nv_bfloat16 ha = __float2bfloat16_rn(ra), hb = __float2bfloat16_rn(rb);
+            oh[at] = ha;
+            oh[at + m / 2] = hb;
+            ol[at] = __float2bfloat16_rn(ra - __bfloat162float(ha));
+            ol[at + m / 2] = __float2bfloat16_rn(rb - __bfloat162float(hb));
+        }
     }
     __nv_bfloat16* kc = second ? p.k2c : p.k1c;
-    for (int g = grp; g < p.n_kv; g += 2) {
-        const float* src = row + static_cast<int64_t>(p.n_q + g) * p.hd;
-        const float a = src[ia], b = src[ib];
-        __nv_bfloat16* dst = kc + (g * p.cap + pos) * m + pi;
-        dst[0] = __float2bfloat16_rn(a * cs - b * sn);
-        dst[m / 2] = __float2bfloat16_rn(a * sn + b * cs);
-        const float2 v = *reinterpret_cast<const float2*>(row + static_cast<int64_t>(p.n_q + p.n_kv + g) * p.hd + 2 * pr);
-        *reinterpret_cast<__nv_bfloat162*>(p.vc + (g * p.cap + pos) * p.hd + 2 * pr) = __floats2bfloat162_rn(v.x, v.y);
+    for (int g0 = grp; g0 < p.n_kv; g0 += 8) {
+        float a[4], b[4];
+        float2 v[4];
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+            const int g = min(g0 + 2 * u, p.n_kv - 1);
+            a[u] = __ldg(row + (p.n_q + g) * p.hd + ia);
+            b[u] = __ldg(row + (p.n_q + g) * p.hd + ib);
+            v[u] = __ldg(reinterpret_cast<const float2*>(row + (p.n_q + p.n_kv + g) * p.hd + 2 * pr));
+        }
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+            const int g = g0 + 2 * u;
+            if (g >= p.n_kv) break;
+            __nv_bfloat16* dst = kc + (g * p.cap + pos) * m + pi;
+            dst[0] = __float2bfloat16_rn(a[u] * cs - b[u] * sn);
+            dst[m / 2] = __float2bfloat16_rn(a[u] * sn + b[u] * cs);
+            *reinterpret_cast<__nv_bfloat162*>(p.vc + (g * p.cap + pos) * p.hd + 2 * pr) = __floats2bfloat162_rn(v[u].x, v[u].y);
+        }
     }
 }
 
@@ -469,14 +521,23 @@ SpanLayout span_layout(int64_t T, int64_t d, int64_t d_ff, int64_t n_q, int64_t 
     return l;
 }
 
+// Pieces of the K range of a product that is added into an addend: while the tiles are fewer than the SMs (a short span's output
+// projection and V product: 18 row tiles at the 2B shape; 130 tokens, V 75 -> 20 us, the call 0.65 -> 0.48 ms), not below eight K chunks a piece.
+int span_split(const spark_ctx* ctx, int64_t rows, int64_t T, int64_t K) {
+    const int64_t tiles = (rows + 127) / 128 * ((T + kSpanTile - 1) / kSpanTile), call = (K + kChunk - 1) / kChunk;
+    int64_t s = ctx->num_sms / tiles;
+    if (s > call / 8) s = call / 8;
+    return s < 1 ? 1 : static_cast<int>(s);
+}
+
 // X operand and weights of one product.
 template <bool MN, bool U>
 int span_gemm(spark_ctx* ctx, SpanGemm p, const void* W, int64_t K, const __nv_bfloat16* X, int64_t ldx, int64_t Tp, cudaStream_t stream) {
-    const int tiles_m = (p.rows + 127) / 128;
     p.call = static_cast<int>((K + kChunk - 1) / kChunk);
-    p.nseg = U ? 1 : (p.call + kSpanSeg - 1) / kSpanSeg;
     p.tiles_t = static_cast<int>((p.T + kSpanTile - 1) / kSpanTile);
-    p.tiles = tiles_m * p.tiles_t;
+    if (p.split < 1) p.split = 1;
+    p.nseg = U ? 1 : ((p.call + p.split - 1) / p.split + kSpanSeg - 1) / kSpanSeg;
+    p.tiles = (p.rows + 127) / 128 * p.tiles_t * p.split;
     p.lo_row = static_cast<int>(Tp);
     p.hdr = ctx->hdr;
     CUtensorMap m_w, m_x;
@@ -541,8 +602,9 @@ int span_layer_launch(spark_ctx* ctx, const spark_layer_weights* w, const spark_
     float* S = reinterpret_cast<float*>(base + l.S);
     __nv_bfloat16* u = reinterpret_cast<__nv_bfloat16*>(base + l.u);
 
-    auto prep = [&](const float* x, const float* norm_w, const float* div, int64_t n, int64_t group) -> int {
-        SpanPrep p{x, norm_w, cfg->rms_eps, div, static_cast<int>(n), static_cast<int>(group), static_cast<int>(l.Tp), xs};
+    const int split_o = span_split(ctx, d, T, nqo), split_v = span_split(ctx, d, T, d_ff);
+    auto prep = [&](const float* x, const float* norm_w, const float* div, int64_t n, int64_t group, float* copy) -> int {
+        SpanPrep p{x, norm_w, cfg->rms_eps, div, static_cast<int>(n), static_cast<int>(group), static_cast<int>(l.Tp), xs, copy};
         void* args[] = {&p};
         return launch_kernel(ctx, reinterpret_cast<const void*>(span_prep_kernel), static_cast<unsigned>(T), 256, 0, stream, false, args, true) == cudaSuccess ? SPARK_OK : SPARK_ERR_CUDA;
     };
@@ -552,7 +614,7 @@ int span_layer_launch(spark_ctx* ctx, const spark_layer_weights* w, const spark_
         g.rows = static_cast<int>(rows); g.add = add; g.y = y;
         return span_gemm<false, false>(ctx, g, W, K, xs, K, l.Tp, stream);
     };
-    int rc = prep(h, w->norm1, nullptr, d, 1);
+    int rc = prep(h, w->norm1, nullptr, d, 1, split_o > 1 ? h2 : nullptr);
     if (rc == SPARK_OK) rc = product(nqkv, w->Wqkv, d, nullptr, qkv);
     if (rc != SPARK_OK) return rc;
 
@@ -582,9 +644,11 @@ int span_layer_launch(spark_ctx* ctx, const spark_layer_weights* w, const spark_
         if (launch_kernel(ctx, reinterpret_cast<const void*>(span_rope_kernel), static_cast<unsigned>(T), 256, 0, stream, false, args, true) != cudaSuccess) return SPARK_ERR_CUDA;
     }
     rc = attn_span_launch(ctx, a, stream);
-    if (rc == SPARK_OK) rc = prep(ao, nullptr, lsum, nqo, hd);
+    if (rc == SPARK_OK) rc = prep(ao, nullptr, lsum, nqo, hd, nullptr);
+    g.split = split_o;
     if (rc == SPARK_OK) rc = product(d, w->Wo, nqo, h, h2);
-    if (rc == SPARK_OK) rc = prep(h2, w->norm2, nullptr, d, 1);
+    g.split = 1;
+    if (rc == SPARK_OK) rc = prep(h2, w->norm2, nullptr, d, 1, split_v > 1 ? h : nullptr);
     if (rc != SPARK_OK) return rc;
 
     g.rows = static_cast<int>(d_ff); g.add = nullptr; g.y = S;
@@ -604,7 +668,7 @@ int span_layer_launch(spark_ctx* ctx, const spark_layer_weights* w, const spark_
     g.S = S; g.theta = theta; g.identity = identity; g.erf_form = (cfg->flags & SPARK_GELU_ERF) ? 1 : 0; g.u = u;
     rc = span_gemm<false, true>(ctx, g, w->K2t, d - cfg->r_ff, xs + cfg->r_ff, d, l.Tp, stream);
     if (rc != SPARK_OK) return rc;
-    g.rows = static_cast<int>(d); g.add = h2; g.y = h;
+    g.rows = static_cast<int>(d); g.add = h2; g.y = h; g.split = split_v;
     return span_gemm<true, false>(ctx, g, w->Vt, d_ff, u, d_ff, l.Tp, stream);
 }
 
