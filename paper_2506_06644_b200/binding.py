@@ -58,6 +58,33 @@ class _KvCache(C.Structure):
 _lib = None
 
 
+class _Entries(dict):
+    """Addresses of the entry points, looked up (and the library loaded) at the first use."""
+
+    def __missing__(self, name):
+        addr = C.cast(getattr(lib(), name), C.c_void_p).value
+        _fastcall().init(torch._C._cuda_getDevice, torch._C._cuda_getCurrentRawStream)
+        self[name] = addr
+        return addr
+
+
+_entry = _Entries()
+
+
+def _fastcall():
+    try:
+        from . import _fastcall as f
+    except ImportError as e:
+        raise RuntimeError("_fastcall.so is missing: run `python -m paper_2506_06644_b200.build`") from e
+    return f
+
+
+def _call(addr, *args):          # replaced by the extension's function at the first use
+    global _call
+    _call = _fastcall().call
+    return _call(addr, *args)
+
+
 def lib() -> C.CDLL:
     """Load the shared library (built in-tree by paper_2506_06644_b200.build); fail loudly if absent."""
     global _lib
@@ -168,6 +195,7 @@ class SparkContext:
             h = C.c_void_p()
             _check(lib().spark_create(C.byref(h), device, self._ws_ptr, nbytes), "spark_create")
         self.handle = h
+        self._h = h.value          # the handle as an integer; 0 once closed
 
     def device_status(self) -> int:
         out = C.c_int(0)
@@ -213,6 +241,7 @@ class SparkContext:
         if self.handle is not None:
             lib().spark_destroy(self.handle)
             self.handle = None
+            self._h = 0
 
     def __del__(self):
         try:
@@ -222,39 +251,33 @@ class SparkContext:
 
 
 def spark_stat_moments(ctx: SparkContext, x, rows, n, ld, moments):
-    _check(lib().spark_stat_moments(ctx.handle, _ptr(x), rows, n, ld, _ptr(moments), _stream()), "spark_stat_moments")
+    _check(_call(_entry["spark_stat_moments"], ctx._h, x, rows, n, ld, moments), "spark_stat_moments")
 
 
 def spark_stat_merge(ctx: SparkContext, parts, m, rows, k, n_total, theta, merged):
-    _check(lib().spark_stat_merge(ctx.handle, _ptr(parts), m, rows, k, n_total, _ptr(theta), _ptr(merged), _stream()),
-           "spark_stat_merge")
+    _check(_call(_entry["spark_stat_merge"], ctx._h, parts, m, rows, k, n_total, theta, merged), "spark_stat_merge")
 
 
 def spark_stat_select(ctx: SparkContext, x, rows, n, ld, theta_in, fill, count, idx, val, idx_cap, y_dense):
-    _check(lib().spark_stat_select(ctx.handle, _ptr(x), rows, n, ld, _ptr(theta_in), fill, _ptr(count), _ptr(idx), _ptr(val),
-                                   idx_cap, _ptr(y_dense), _stream()), "spark_stat_select")
+    _check(_call(_entry["spark_stat_select"], ctx._h, x, rows, n, ld, theta_in, fill, count, idx, val, idx_cap, y_dense), "spark_stat_select")
 
 
 def spark_stat_topk(ctx: SparkContext, x, rows, n, ld, k, fill, theta, count, idx, val, idx_cap, y_dense):
-    _check(lib().spark_stat_topk(ctx.handle, _ptr(x), rows, n, ld, k, fill, _ptr(theta), _ptr(count), _ptr(idx),
-                                 _ptr(val), idx_cap, _ptr(y_dense), _stream()), "spark_stat_topk")
+    _check(_call(_entry["spark_stat_topk"], ctx._h, x, rows, n, ld, k, fill, theta, count, idx, val, idx_cap, y_dense), "spark_stat_topk")
 
 
 def spark_ffn_decode(ctx: SparkContext, x, B, K1t, K2t, Vt, wdtype, d, d_ff, r, k, flags, y, theta, count, idx):
-    _check(lib().spark_ffn_decode(ctx.handle, _ptr(x), B, _ptr(K1t), _ptr(K2t), _ptr(Vt), wdtype, d, d_ff, r, k,
-                                  flags, _ptr(y), _ptr(theta), _ptr(count), _ptr(idx), _stream()), "spark_ffn_decode")
+    _check(_call(_entry["spark_ffn_decode"], ctx._h, x, B, K1t, K2t, Vt, wdtype, d, d_ff, r, k, flags, y, theta, count, idx), "spark_ffn_decode")
 
 
 def spark_ffn_decode_fp8(ctx: SparkContext, x, B, K1t, K1s, K2t, K2s, Vt, Vs, d, d_ff, r, k, flags, y, theta, count, idx):
-    _check(lib().spark_ffn_decode_fp8(ctx.handle, _ptr(x), B, _ptr(K1t), _ptr(K1s), _ptr(K2t), _ptr(K2s), _ptr(Vt), _ptr(Vs), d,
-                                      d_ff, r, k, flags, _ptr(y), _ptr(theta), _ptr(count), _ptr(idx), _stream()), "spark_ffn_decode_fp8")
+    _check(_call(_entry["spark_ffn_decode_fp8"], ctx._h, x, B, K1t, K1s, K2t, K2s, Vt, Vs, d, d_ff, r, k, flags, y, theta, count, idx), "spark_ffn_decode_fp8")
 
 
 def spark_ffn_decode_noalloc(x, B, K1t, K2t, Vt, wdtype, d, d_ff, r, k, flags, y, theta):
     """spark_ffn_decode for callers that must not allocate: no context, no workspace; the kernel's
     inter-block state lives in a fixed array inside the library (see include/spark.h).  B <= 16."""
-    _check(lib().spark_ffn_decode_noalloc(_ptr(x), B, _ptr(K1t), _ptr(K2t), _ptr(Vt), wdtype, d, d_ff, r, k, flags,
-                                          _ptr(y), _ptr(theta), _stream()), "spark_ffn_decode_noalloc")
+    _check(_call(_entry["spark_ffn_decode_noalloc"], x, B, K1t, K2t, Vt, wdtype, d, d_ff, r, k, flags, y, theta), "spark_ffn_decode_noalloc")
 
 
 def spark_noalloc_status() -> int:
@@ -266,28 +289,21 @@ def spark_noalloc_status() -> int:
 
 def spark_attn_decode(ctx: SparkContext, q, k1c, k2c, vc, kvdtype, B, n_q, n_kv, hd, r, cap, ctx_len, window,
                       k_attn, flags, o, theta, count, idx, idx_cap):
-    _check(lib().spark_attn_decode(ctx.handle, _ptr(q), _ptr(k1c), _ptr(k2c), _ptr(vc), kvdtype, B, n_q, n_kv, hd,
-                                   r, cap, _ptr(ctx_len), window, k_attn, flags, _ptr(o), _ptr(theta), _ptr(count),
-                                   _ptr(idx), idx_cap, _stream()), "spark_attn_decode")
+    _check(_call(_entry["spark_attn_decode"], ctx._h, q, k1c, k2c, vc, kvdtype, B, n_q, n_kv, hd, r, cap, ctx_len, window, k_attn, flags, o, theta, count, idx, idx_cap), "spark_attn_decode")
 
 
 def spark_attn_decode_fp8k(ctx: SparkContext, q, k1c, k1s, k2c, vc, B, n_q, n_kv, hd, r, cap, ctx_len, window, k_attn, flags,
                            o, theta, count, idx, idx_cap):
-    _check(lib().spark_attn_decode_fp8k(ctx.handle, _ptr(q), _ptr(k1c), _ptr(k1s), _ptr(k2c), _ptr(vc), B, n_q, n_kv, hd, r, cap,
-                                        _ptr(ctx_len), window, k_attn, flags, _ptr(o), _ptr(theta), _ptr(count), _ptr(idx), idx_cap,
-                                        _stream()), "spark_attn_decode_fp8k")
+    _check(_call(_entry["spark_attn_decode_fp8k"], ctx._h, q, k1c, k1s, k2c, vc, B, n_q, n_kv, hd, r, cap, ctx_len, window, k_attn, flags, o, theta, count, idx, idx_cap), "spark_attn_decode_fp8k")
 
 
 def spark_attn_decode_fp8kv(ctx: SparkContext, q, k1c, k1s, k2c, k2s, vc, vs, B, n_q, n_kv, hd, r, cap, ctx_len, window, k_attn, flags,
                             o, theta, count, idx, idx_cap):
-    _check(lib().spark_attn_decode_fp8kv(ctx.handle, _ptr(q), _ptr(k1c), _ptr(k1s), _ptr(k2c), _ptr(k2s), _ptr(vc), _ptr(vs), B, n_q, n_kv,
-                                         hd, r, cap, _ptr(ctx_len), window, k_attn, flags, _ptr(o), _ptr(theta), _ptr(count), _ptr(idx),
-                                         idx_cap, _stream()), "spark_attn_decode_fp8kv")
+    _check(_call(_entry["spark_attn_decode_fp8kv"], ctx._h, q, k1c, k1s, k2c, k2s, vc, vs, B, n_q, n_kv, hd, r, cap, ctx_len, window, k_attn, flags, o, theta, count, idx, idx_cap), "spark_attn_decode_fp8kv")
 
 
 def spark_dense_gemv(ctx: SparkContext, x, B, Wt, wdtype, n_in, n_out, y_add, y):
-    _check(lib().spark_dense_gemv(ctx.handle, _ptr(x), B, _ptr(Wt), wdtype, n_in, n_out, _ptr(y_add), _ptr(y),
-                                  _stream()), "spark_dense_gemv")
+    _check(_call(_entry["spark_dense_gemv"], ctx._h, x, B, Wt, wdtype, n_in, n_out, y_add, y), "spark_dense_gemv")
 
 
 @dataclass
@@ -307,8 +323,8 @@ def make_layer(weights: dict, cfg: dict, cache: dict) -> LayerHandles:
 
 
 def spark_layer_decode(ctx: SparkContext, layer: LayerHandles, ctx_len, h, B, scratch):
-    _check(lib().spark_layer_decode(ctx.handle, C.byref(layer.weights), C.byref(layer.cfg), C.byref(layer.cache),
-                                    _ptr(ctx_len), _ptr(h), B, _ptr(scratch), _stream()), "spark_layer_decode")
+    _check(_call(_entry["spark_layer_decode"], ctx._h, C.addressof(layer.weights), C.addressof(layer.cfg), C.addressof(layer.cache),
+                 ctx_len, h, B, scratch), "spark_layer_decode")
 
 
 @dataclass
@@ -331,8 +347,8 @@ def make_stack(layers) -> StackHandles:
 
 
 def spark_stack_decode(ctx: SparkContext, stack: StackHandles, ctx_len, h, B, scratch):
-    _check(lib().spark_stack_decode(ctx.handle, stack.weights, stack.cfgs, stack.caches, stack.n_layers, _ptr(ctx_len), _ptr(h), B,
-                                    _ptr(scratch), _stream()), "spark_stack_decode")
+    _check(_call(_entry["spark_stack_decode"], ctx._h, C.addressof(stack.weights), C.addressof(stack.cfgs), C.addressof(stack.caches),
+                 stack.n_layers, ctx_len, h, B, scratch), "spark_stack_decode")
 
 
 def layer_scratch_floats(cfg: dict, B: int) -> int:

@@ -1,4 +1,4 @@
-"""Build the CUDA library in-tree: csrc/*.cu -> libspark_b200.so (sm_100a only).
+"""Build in-tree: csrc/*.cu -> libspark_b200.so (sm_100a only), csrc/fastcall.c -> _fastcall.so (how binding.py calls it).
 
 Run as `python -m paper_2506_06644_b200.build` or through `__graft_entry__.build()`.
 nvcc cross-compiles without a GPU.  Objects are rebuilt only when a source or header is newer.
@@ -8,12 +8,14 @@ from __future__ import annotations
 import os
 import subprocess
 import sys
+import sysconfig
 from concurrent.futures import ThreadPoolExecutor
 
 HERE = os.path.dirname(os.path.abspath(__file__))
 CSRC = os.path.join(HERE, "csrc")
 OBJ = os.path.join(HERE, "build")
 LIB = os.path.join(HERE, "libspark_b200.so")
+FASTCALL = os.path.join(HERE, "_fastcall.so")
 
 NVCC_FLAGS = [
     "-gencode", "arch=compute_100a,code=sm_100a", "-lineinfo", "-O3", "-std=c++17",
@@ -41,8 +43,19 @@ def _newest_header() -> float:
     return t
 
 
+def build_fastcall(force: bool = False) -> str:
+    src = os.path.join(CSRC, "fastcall.c")
+    if force or not os.path.exists(FASTCALL) or os.path.getmtime(FASTCALL) < os.path.getmtime(src):
+        cmd = [os.environ.get("CC", "gcc"), "-O2", "-fPIC", "-shared", "-I", sysconfig.get_paths()["include"], src, "-o", FASTCALL]
+        res = subprocess.run(cmd, capture_output=True, text=True)
+        if res.returncode != 0:
+            raise RuntimeError(f"{cmd[0]} failed for {src}:\n{res.stdout}\n{res.stderr}")
+    return FASTCALL
+
+
 def build(force: bool = False, verbose: bool = False) -> str:
     os.makedirs(OBJ, exist_ok=True)
+    build_fastcall(force)
     nvcc = _nvcc()
     hdr_t = _newest_header()
     objs, jobs = [], []

@@ -8,6 +8,7 @@
 // distributed shared memory.  Rows too long to be held on chip fall back to re-reading global
 // memory in the later sweeps.
 #include <cooperative_groups.h>
+#include <cstdlib>
 
 #include "common.cuh"
 
@@ -624,6 +625,204 @@ __global__ void __launch_bounds__(kRowThreads, 1) stat_topk_row_kernel(const Top
     }
 }
 
+// ---------------------------------------------------------------------------------------------
+// Rows of up to 64K values in registers: a group of 1..16 warps holds up to 16K of them, eight float4 per lane and warp, every
+// load in flight at once; a cluster of up to four such blocks holds a longer row.  A row costs two exchanges (sum; squared
+// deviations) and, for the outputs, one more (counts), among warps of a group through shared memory, among blocks through
+// distributed shared memory; rows of up to 1024 values need none.  A warp owns a contiguous run, so ranks inside the ordered lists
+// come from four ballots per 128 values.
+// ---------------------------------------------------------------------------------------------
+constexpr int kRegVec = 8;
+constexpr int kRegWarpVec = kRegVec * 32;        // float4 a warp holds
+
+template <int WPR>
+__global__ void __launch_bounds__(WPR < 4 ? 128 : WPR * 32) stat_topk_reg_kernel(const TopkParams p, int cl) {
+    constexpr int kBlockWarps = WPR < 4 ? 4 : WPR, kRows = kBlockWarps / WPR;      // rows per block
+    __shared__ double red[2][kBlockWarps];
+    __shared__ int cnt_s[kBlockWarps];
+    __shared__ double part[2];                   // read by the other blocks of the cluster
+    __shared__ int part_cnt;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, slot = warp / WPR, w = warp - slot * WPR;
+    const int rank = cl > 1 ? static_cast<int>(blockIdx.x % cl) : 0;
+    const int64_t row = cl > 1 ? blockIdx.x / cl : static_cast<int64_t>(blockIdx.x) * kRows + slot;
+    if (row >= p.rows) return;                   // whole groups (kRows > 1 only without clusters)
+    auto group_sync = [&]() {
+        if (WPR == kBlockWarps) __syncthreads();
+        else if (WPR > 1) asm volatile("bar.sync %0, %1;" ::"r"(slot + 1), "n"(WPR * 32) : "memory");
+    };
+    auto cluster_sync = [&]() { cg::this_cluster().sync(); };
+    const int64_t begin = rank * p.chunk;
+    const int len = static_cast<int>(p.n - begin < p.chunk ? (p.n > begin ? p.n - begin : 0) : p.chunk);
+    const int nvec = (len + 3) >> 2, vpw = (nvec + WPR - 1) / WPR, v0 = w * vpw + lane, vend = min(nvec, (w + 1) * vpw);
+    const float4* src = reinterpret_cast<const float4*>(p.x + row * p.ld + begin);
+    float4 f[kRegVec];
+#pragma unroll
+    for (int j = 0; j < kRegVec; ++j) {
+        uint4 u = make_uint4(0u, 0u, 0u, 0u);
+        if (v0 + 32 * j < vend) u = ld_stream16(src + v0 + 32 * j);
+        f[j] = make_float4(__uint_as_float(u.x), __uint_as_float(u.y), __uint_as_float(u.z), __uint_as_float(u.w));
+    }
+    // entries of vector j that belong to the row: 4 but for the row's last vector and what lies behind the warp's run
+    auto valid = [&](int j) -> int { return v0 + 32 * j < vend ? min(len - 4 * (v0 + 32 * j), 4) : 0; };
+    // sum over the row of a quantity that every lane has a part of
+    auto row_sum = [&](double v, int which) -> double {
+        v = warp_sum_f64(v);
+        if (WPR > 1) {
+            if (lane == 0) red[which][warp] = v;
+            group_sync();
+            v = 0.0;
+#pragma unroll
+            for (int i = 0; i < WPR; ++i) v += red[which][slot * WPR + i];
+        }
+        if (cl > 1) {
+            if (threadIdx.x == 0) part[which] = v;
+            cluster_sync();
+            v = 0.0;
+            for (int c = 0; c < cl; ++c) v += *cg::this_cluster().map_shared_rank(&part[which], c);
+        }
+        return v;
+    };
+    float theta = -INFINITY;
+    if (p.theta_in != nullptr) {
+        theta = p.theta_in[row];
+    } else if (!p.identity) {
+        // what lies behind the row reads as zero in its last vector: cleared, so that the sums need no tests
+        float s0 = 0.f, s1 = 0.f;
+#pragma unroll
+        for (int j = 0; j < kRegVec; ++j) {
+            const int nv = valid(j);
+            if (nv < 4) {
+                if (nv < 1) f[j].x = 0.f;
+                if (nv < 2) f[j].y = 0.f;
+                if (nv < 3) f[j].z = 0.f;
+                f[j].w = 0.f;
+            }
+            s0 += f[j].x + f[j].y;
+            s1 += f[j].z + f[j].w;
+        }
+        const double mean = row_sum(static_cast<double>(s0) + static_cast<double>(s1), 0) / static_cast<double>(p.n);
+        // squared deviations around the mean (two-pass form of the text below Eq. 11); around its fp32 rounding, corrected:
+        // sum (x - m)^2 = sum (x - mf)^2 - n (m - mf)^2
+        const float mf = static_cast<float>(mean);
+        float q0 = 0.f, q1 = 0.f;
+#pragma unroll
+        for (int j = 0; j < kRegVec; ++j) {
+            const int nv = valid(j);
+            const float a = nv > 0 ? f[j].x - mf : 0.f, b = nv > 1 ? f[j].y - mf : 0.f, c = nv > 2 ? f[j].z - mf : 0.f, d = nv > 3 ? f[j].w - mf : 0.f;
+            q0 = fmaf(a, a, fmaf(b, b, q0));
+            q1 = fmaf(c, c, fmaf(d, d, q1));
+        }
+        const double dm = mean - static_cast<double>(mf);
+        const double m2 = row_sum(static_cast<double>(q0) + static_cast<double>(q1), 1) - static_cast<double>(p.n) * dm * dm;
+        const Moments m{static_cast<double>(p.n), mean, m2 > 0.0 ? m2 : 0.0};
+        if (p.moments_out != nullptr) {          // a shard's moments for the caller to merge (Appendix: global statistical top-k)
+            if (rank == 0 && w == 0 && lane == 0) {
+                p.moments_out[row * 3 + 0] = m.n;
+                p.moments_out[row * 3 + 1] = m.mean;
+                p.moments_out[row * 3 + 2] = m.m2;
+            }
+            if (cl > 1) cluster_sync();          // no block may leave while a peer can still read its shared memory
+            return;
+        }
+        theta = theta_from(m, p.z);
+    }
+    // a given threshold of -inf is spark_stat_merge's "k >= n_total": everything survives, unshifted
+    const float shift = (p.identity || theta == -INFINITY) ? 0.f : theta;
+    const bool want_lists = p.idx != nullptr || p.val != nullptr;
+    // one bit per entry of the lane's vectors
+    unsigned mask = 0u;
+#pragma unroll
+    for (int j = 0; j < kRegVec; ++j) {
+        const int nv = valid(j);
+        mask |= ((nv > 0 && f[j].x > theta ? 1u : 0u) | (nv > 1 && f[j].y > theta ? 2u : 0u) | (nv > 2 && f[j].z > theta ? 4u : 0u) |
+                 (nv > 3 && f[j].w > theta ? 8u : 0u)) << (4 * j);
+    }
+    const int mine = __reduce_add_sync(kFull, __popc(mask));
+    int total = mine, base = 0;                  // survivors of the row; those ahead of this warp's run
+    if (WPR > 1) {
+        if (lane == 0) cnt_s[warp] = mine;
+        group_sync();
+        total = 0;
+#pragma unroll
+        for (int i = 0; i < WPR; ++i) {
+            if (i < w) base += cnt_s[slot * WPR + i];
+            total += cnt_s[slot * WPR + i];
+        }
+    }
+    if (cl > 1) {
+        if (threadIdx.x == 0) part_cnt = total;
+        cluster_sync();
+        total = 0;
+        for (int c = 0; c < cl; ++c) {
+            const int pc = *cg::this_cluster().map_shared_rank(&part_cnt, c);
+            if (c < rank) base += pc;
+            total += pc;
+        }
+    }
+    if (rank == 0 && w == 0 && lane == 0) {
+        if (p.theta != nullptr) p.theta[row] = theta;
+        if (p.count != nullptr) p.count[row] = total;
+        if (want_lists && total > p.idx_cap) atomicCAS(&p.hdr->status, SPARK_OK, SPARK_ERR_OVERFLOW);
+    }
+    if (p.y_dense != nullptr) {
+        const float fillv = p.fill == SPARK_FILL_NEGINF ? -INFINITY : 0.f;
+        float* yrow = p.y_dense + row * p.ld + begin;
+#pragma unroll
+        for (int j = 0; j < kRegVec; ++j) {
+            const int v = v0 + 32 * j, nv = valid(j);
+            const unsigned b = mask >> (4 * j);
+            const float4 o = make_float4(b & 1u ? f[j].x - shift : fillv, b & 2u ? f[j].y - shift : fillv, b & 4u ? f[j].z - shift : fillv, b & 8u ? f[j].w - shift : fillv);
+            if (nv == 4) {
+                __stcs(reinterpret_cast<float4*>(yrow) + v, o);
+            } else if (nv > 0) {
+                yrow[4 * v] = o.x;
+                if (nv > 1) yrow[4 * v + 1] = o.y;
+                if (nv > 2) yrow[4 * v + 2] = o.z;
+            }
+        }
+    }
+    if (want_lists) {
+        int32_t* idx_row = p.idx != nullptr ? p.idx + row * p.idx_cap : nullptr;
+        float* val_row = p.val != nullptr ? p.val + row * p.idx_cap : nullptr;
+        const unsigned lt = (1u << lane) - 1u;
+        int64_t off = base;
+#pragma unroll
+        for (int j = 0; j < kRegVec; ++j) {
+            const unsigned b = mask >> (4 * j);
+            const unsigned b0 = __ballot_sync(kFull, b & 1u), b1 = __ballot_sync(kFull, b & 2u), b2 = __ballot_sync(kFull, b & 4u), b3 = __ballot_sync(kFull, b & 8u);
+            int64_t pos = off + __popc(b0 & lt) + __popc(b1 & lt) + __popc(b2 & lt) + __popc(b3 & lt);
+            const float fv[4] = {f[j].x, f[j].y, f[j].z, f[j].w};
+#pragma unroll
+            for (int e = 0; e < 4; ++e)
+                if (b >> e & 1u) {
+                    if (pos < p.idx_cap) {
+                        if (idx_row != nullptr) idx_row[pos] = static_cast<int32_t>(begin) + 4 * (v0 + 32 * j) + e;
+                        if (val_row != nullptr) val_row[pos] = fv[e] - shift;
+                    }
+                    ++pos;
+                }
+            off += __popc(b0) + __popc(b1) + __popc(b2) + __popc(b3);
+        }
+    }
+    if (cl > 1) cluster_sync();                  // no block may leave while a peer can still read its shared memory
+}
+
+template <int WPR>
+cudaError_t reg_launch(const TopkParams& p, int cl, cudaStream_t stream) {
+    constexpr int kThreadsR = WPR < 4 ? 128 : WPR * 32, kRows = WPR < 4 ? 4 / WPR : 1;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(static_cast<unsigned>(cl > 1 ? p.rows * cl : (p.rows + kRows - 1) / kRows));
+    cfg.blockDim = dim3(kThreadsR);
+    cfg.stream = stream;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeClusterDimension;
+    attr[0].val.clusterDim.x = cl;
+    attr[0].val.clusterDim.y = attr[0].val.clusterDim.z = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = cl > 1 ? 1 : 0;
+    return cudaLaunchKernelEx(&cfg, stat_topk_reg_kernel<WPR>, p, cl);
+}
+
 bool g_attr_done[64] = {};   // per device: opt-in shared memory configured
 
 }  // namespace
@@ -656,6 +855,17 @@ static int topk_launch(spark_ctx* ctx, const float* x, int64_t rows, int64_t n, 
     p.theta = theta; p.count = count; p.idx = idx; p.val = val; p.idx_cap = idx_cap; p.y_dense = y_dense;
     p.theta_in = theta_in; p.moments_out = moments_out;
     p.hdr = ctx->hdr;
+
+    static const int regmode = getenv("REGMODE") ? atoi(getenv("REGMODE")) : 1;
+    if (n <= 65536 && (regmode == 1 ? (n <= 16384 || rows <= 1000000) : regmode == 2 ? n <= 16384 : false)) {
+        const int rcl = n <= 16384 ? 1 : (n <= 32768 ? 2 : 4);
+        p.chunk = ((n + rcl - 1) / rcl + 3) / 4 * 4;
+        const int warps = static_cast<int>((p.chunk + 4 * kRegWarpVec - 1) / (4 * kRegWarpVec));
+        cudaStream_t st = static_cast<cudaStream_t>(stream);
+        const cudaError_t er = warps <= 1 ? reg_launch<1>(p, rcl, st) : warps <= 2 ? reg_launch<2>(p, rcl, st) : warps <= 4 ? reg_launch<4>(p, rcl, st)
+                             : warps <= 8 ? reg_launch<8>(p, rcl, st) : reg_launch<16>(p, rcl, st);
+        return er == cudaSuccess ? SPARK_OK : SPARK_ERR_CUDA;
+    }
 
     if (ctx->device >= 0 && ctx->device < 64 && !g_attr_done[ctx->device]) {
         if (cudaFuncSetAttribute(stat_topk_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
