@@ -1,14 +1,12 @@
 // spark_stat_topk: standalone statistical top-k over many rows (Section 3, Eq. 9-11).
 //
-// Two kernels.  Rows of 16K..64K values: one persistent block per SM holds a whole row on chip
-// (stat_topk_row_kernel below).  All other lengths: one thread-block cluster per row; each block
-// of the cluster streams its contiguous part of the row from HBM exactly once into shared memory,
-// and every later sweep (squared deviations around the exact mean, counting, ordered compaction /
-// dense output) reads shared memory.  Partial sums travel between the blocks of a cluster through
-// distributed shared memory.  Rows too long to be held on chip fall back to re-reading global
-// memory in the later sweeps.
+// Three kernels; the dispatch at the end says which serves what.  Short rows (and the lists of few longer ones): in registers,
+// one to sixteen warps per row (stat_topk_reg_kernel).  Rows of 16K..64K values: one persistent block per SM holds a whole row on
+// chip (stat_topk_row_kernel).  All other lengths: one thread-block cluster per row; each block of the cluster streams its
+// contiguous part of the row from HBM exactly once into shared memory, and every later sweep (squared deviations around the exact
+// mean, counting, ordered compaction / dense output) reads shared memory.  Partial sums travel between the blocks of a cluster
+// through distributed shared memory.  Rows too long to be held on chip fall back to re-reading global memory in the later sweeps.
 #include <cooperative_groups.h>
-#include <cstdlib>
 
 #include "common.cuh"
 
@@ -25,6 +23,7 @@ struct TopkParams {
     int64_t rows, n, ld, k;
     int64_t chunk;        // elements per block (multiple of 4)
     int fill;
+    int direct;           // row kernel: lists by ballots instead of staging windows
     int identity;         // k >= n: keep everything unshifted
     double z;             // Q(1 - k/n)
     float* theta;
@@ -329,6 +328,7 @@ struct RowShared {
 };
 
 // One row: cur holds its register part, nxt receives the next row's.  Returns false after a timeout.
+template <bool LISTS>
 __device__ __forceinline__ bool row_body(const TopkParams& p, const RowGeom& g, float* srow, RowShared& sh, int64_t row, int64_t next_row,
                                          uint32_t parity, uint4 (&cur)[kRowRegVec], uint4 (&nxt)[kRowRegVec], float c, float& c_next) {
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
@@ -402,6 +402,56 @@ __device__ __forceinline__ bool row_body(const TopkParams& p, const RowGeom& g, 
     }
     const float shift = p.identity ? 0.f : theta;
 
+    // ---- no lists: survivors counted and the dense result written in one sweep ------------------------------
+    // (a separate counting sweep that leaves bits cost four instructions per value and a second read of shared memory:
+    // 4096 x 65536, dense result 444 -> 370 us = 5.8 TB/s, statistics 240 -> 222)
+    if constexpr (!LISTS) {
+        const float fillv = p.fill == SPARK_FILL_NEGINF ? -INFINITY : 0.f;
+        float* yrow = p.y_dense != nullptr ? p.y_dense + row * p.ld : nullptr;
+        int cnt = 0;
+        auto take = [&](const float4& f, int v) {
+            const bool a0 = f.x > theta, a1 = f.y > theta, a2 = f.z > theta, a3 = f.w > theta;
+            cnt += a0; cnt += a1; cnt += a2; cnt += a3;
+            if (yrow != nullptr)
+                __stcs(reinterpret_cast<float4*>(yrow) + v, make_float4(a0 ? f.x - shift : fillv, a1 ? f.y - shift : fillv, a2 ? f.z - shift : fillv, a3 ? f.w - shift : fillv));
+        };
+        int v = tid;
+        for (; v + 3 * kRowThreads < g.ns; v += 4 * kRowThreads) {
+            float4 f[4];
+#pragma unroll
+            for (int u = 0; u < 4; ++u) f[u] = ssrc[v + u * kRowThreads];
+#pragma unroll
+            for (int u = 0; u < 4; ++u) take(f[u], v + u * kRowThreads);
+        }
+        for (; v < g.ns; v += kRowThreads) take(ssrc[v], v);
+#pragma unroll
+        for (int i = 0; i < kRowRegVec; ++i) {
+            const int vr = rv0 + i * 32;
+            if (vr >= g.nvec) continue;
+            const float4 f = f4(cur[i]);
+            if (vr < g.nvec - 1 || last_nv == 4) {
+                take(f, vr);
+            } else {
+                const float fv[3] = {f.x, f.y, f.z};
+                for (int e = 0; e < last_nv; ++e) {
+                    cnt += fv[e] > theta;
+                    if (yrow != nullptr) yrow[4 * vr + e] = fv[e] > theta ? fv[e] - shift : fillv;
+                }
+            }
+        }
+        cnt = __reduce_add_sync(kFull, cnt);
+        if (lane == 0) sh.scan[warp] = cnt;
+        __syncthreads();                                              // shared memory is free: the next row's copies
+        if (tid == 0) {
+            if (next_row < p.rows) row_issue_bulk(p.x + next_row * p.ld, srow, sh.mbar, g);
+            int total = 0;
+#pragma unroll
+            for (int w = 0; w < kRowWarps; ++w) total += sh.scan[w];
+            if (p.theta) p.theta[row] = theta;
+            if (p.count) p.count[row] = total;
+        }
+        return true;
+    } else {
     // ---- count: one bit per value of the thread's two runs ------------------------------------------
     unsigned ms[3] = {0u, 0u, 0u};                                    // 92 bits: shared-memory run
     unsigned long long mr = 0ull;                                     // 36 bits: register run
@@ -443,15 +493,50 @@ __device__ __forceinline__ bool row_body(const TopkParams& p, const RowGeom& g, 
     }
     const int excl = base + inc - packed;
     const int tot_s = tot & 0xffff, total = tot_s + (tot >> 16);
-    const bool want_lists = (p.idx != nullptr) || (p.val != nullptr);
     if (tid == 0) {
         if (p.theta) p.theta[row] = theta;
         if (p.count) p.count[row] = total;
-        if (want_lists && total > p.idx_cap) atomicCAS(&p.hdr->status, SPARK_OK, SPARK_ERR_OVERFLOW);
+        if (total > p.idx_cap) atomicCAS(&p.hdr->status, SPARK_OK, SPARK_ERR_OVERFLOW);
     }
 
-    // ---- ordered lists: each warp stages its (contiguous) share in a 256-entry window of its own -------
-    if (want_lists) {
+    // ---- ordered lists ---------------------------------------------------------------------------------
+    if (p.direct) {
+        // many survivors: a warp walks its contiguous vectors 32 at a time, ranks from four ballots, and stores straight into the
+        // lists (neighbouring lanes write neighbouring entries)
+        int32_t* idx_row = p.idx ? p.idx + row * p.idx_cap : nullptr;
+        float* val_row = p.val ? p.val + row * p.idx_cap : nullptr;
+        const unsigned lt = (1u << lane) - 1u;
+        const int cap = static_cast<int>(p.idx_cap < g.n ? p.idx_cap : g.n);
+        auto put = [&](const float4& f, int v, int nv, int& off) {
+            const bool a0 = nv > 0 && f.x > theta, a1 = nv > 1 && f.y > theta, a2 = nv > 2 && f.z > theta, a3 = nv > 3 && f.w > theta;
+            const unsigned b0 = __ballot_sync(kFull, a0), b1 = __ballot_sync(kFull, a1), b2 = __ballot_sync(kFull, a2), b3 = __ballot_sync(kFull, a3);
+            int pos = off + __popc(b0 & lt) + __popc(b1 & lt) + __popc(b2 & lt) + __popc(b3 & lt);
+            auto one = [&](bool on, float x, int e) {
+                if (on) {
+                    if (pos < cap) {
+                        if (idx_row) idx_row[pos] = 4 * v + e;
+                        if (val_row) val_row[pos] = x - shift;
+                    }
+                    ++pos;
+                }
+            };
+            one(a0, f.x, 0); one(a1, f.y, 1); one(a2, f.z, 2); one(a3, f.w, 3);
+            off += __popc(b0) + __popc(b1) + __popc(b2) + __popc(b3);
+        };
+        int off = base & 0xffff;
+#pragma unroll 4
+        for (int i = 0; i < kRowRunVec; ++i) {
+            const int v = warp * 32 * kRowRunVec + 32 * i + lane;
+            put(v < g.ns ? ssrc[v] : make_float4(0.f, 0.f, 0.f, 0.f), v, v < g.ns ? 4 : 0, off);
+        }
+        off = tot_s + (base >> 16);
+#pragma unroll
+        for (int i = 0; i < kRowRegVec; ++i) {
+            const int v = rv0 + 32 * i;
+            put(f4(cur[i]), v, v < g.nvec ? (v == g.nvec - 1 ? last_nv : 4) : 0, off);
+        }
+    } else {
+        // few: each warp stages its (contiguous) share in a 256-entry window of its own
         int* wi = reinterpret_cast<int*>(srow + kRowSmemVec * 4) + warp * (2 * kRowWin);
         float* wv = reinterpret_cast<float*>(wi + kRowWin);
         int32_t* idx_row = p.idx ? p.idx + row * p.idx_cap : nullptr;
@@ -572,8 +657,11 @@ __device__ __forceinline__ bool row_body(const TopkParams& p, const RowGeom& g, 
     __syncthreads();
     if (tid == 0 && next_row < p.rows) row_issue_bulk(p.x + next_row * p.ld, srow, sh.mbar, g);
     return true;
+    }
 }
 
+// LISTS: with index or value lists (and perhaps the dense result); otherwise statistics and the dense result only.
+template <bool LISTS>
 __global__ void __launch_bounds__(kRowThreads, 1) stat_topk_row_kernel(const TopkParams p) {
     extern __shared__ __align__(16) float srow[];
     __shared__ RowShared sh;
@@ -603,11 +691,11 @@ __global__ void __launch_bounds__(kRowThreads, 1) stat_topk_row_kernel(const Top
     uint32_t parity = 0;
 #pragma unroll 1
     for (;;) {
-        ok = row_body(p, g, srow, sh, row, row + step, parity, ra, rb, ca, cb);
+        ok = row_body<LISTS>(p, g, srow, sh, row, row + step, parity, ra, rb, ca, cb);
         row += step;
         if (!ok || row >= p.rows) break;
         parity ^= 1u;
-        ok = row_body(p, g, srow, sh, row, row + step, parity, rb, ra, cb, ca);
+        ok = row_body<LISTS>(p, g, srow, sh, row, row + step, parity, rb, ra, cb, ca);
         row += step;
         if (!ok || row >= p.rows) break;
         parity ^= 1u;
@@ -662,6 +750,8 @@ __global__ void __launch_bounds__(WPR < 4 ? 128 : WPR * 32) stat_topk_reg_kernel
         if (v0 + 32 * j < vend) u = ld_stream16(src + v0 + 32 * j);
         f[j] = make_float4(__uint_as_float(u.x), __uint_as_float(u.y), __uint_as_float(u.z), __uint_as_float(u.w));
     }
+    // vectors j < nfull are whole in every lane of the warp and need no tests
+    const int nfull = (min(vend, len >> 2) - w * vpw) >> 5;
     // entries of vector j that belong to the row: 4 but for the row's last vector and what lies behind the warp's run
     auto valid = [&](int j) -> int { return v0 + 32 * j < vend ? min(len - 4 * (v0 + 32 * j), 4) : 0; };
     // sum over the row of a quantity that every lane has a part of
@@ -690,12 +780,14 @@ __global__ void __launch_bounds__(WPR < 4 ? 128 : WPR * 32) stat_topk_reg_kernel
         float s0 = 0.f, s1 = 0.f;
 #pragma unroll
         for (int j = 0; j < kRegVec; ++j) {
-            const int nv = valid(j);
-            if (nv < 4) {
-                if (nv < 1) f[j].x = 0.f;
-                if (nv < 2) f[j].y = 0.f;
-                if (nv < 3) f[j].z = 0.f;
-                f[j].w = 0.f;
+            if (j >= nfull) {
+                const int nv = valid(j);
+                if (nv < 4) {
+                    if (nv < 1) f[j].x = 0.f;
+                    if (nv < 2) f[j].y = 0.f;
+                    if (nv < 3) f[j].z = 0.f;
+                    f[j].w = 0.f;
+                }
             }
             s0 += f[j].x + f[j].y;
             s1 += f[j].z + f[j].w;
@@ -707,8 +799,14 @@ __global__ void __launch_bounds__(WPR < 4 ? 128 : WPR * 32) stat_topk_reg_kernel
         float q0 = 0.f, q1 = 0.f;
 #pragma unroll
         for (int j = 0; j < kRegVec; ++j) {
-            const int nv = valid(j);
-            const float a = nv > 0 ? f[j].x - mf : 0.f, b = nv > 1 ? f[j].y - mf : 0.f, c = nv > 2 ? f[j].z - mf : 0.f, d = nv > 3 ? f[j].w - mf : 0.f;
+            float a = f[j].x - mf, b = f[j].y - mf, c = f[j].z - mf, d = f[j].w - mf;
+            if (j >= nfull) {
+                const int nv = valid(j);
+                if (nv < 1) a = 0.f;
+                if (nv < 2) b = 0.f;
+                if (nv < 3) c = 0.f;
+                if (nv < 4) d = 0.f;
+            }
             q0 = fmaf(a, a, fmaf(b, b, q0));
             q1 = fmaf(c, c, fmaf(d, d, q1));
         }
@@ -733,9 +831,9 @@ __global__ void __launch_bounds__(WPR < 4 ? 128 : WPR * 32) stat_topk_reg_kernel
     unsigned mask = 0u;
 #pragma unroll
     for (int j = 0; j < kRegVec; ++j) {
-        const int nv = valid(j);
-        mask |= ((nv > 0 && f[j].x > theta ? 1u : 0u) | (nv > 1 && f[j].y > theta ? 2u : 0u) | (nv > 2 && f[j].z > theta ? 4u : 0u) |
-                 (nv > 3 && f[j].w > theta ? 8u : 0u)) << (4 * j);
+        unsigned nib = (f[j].x > theta ? 1u : 0u) | (f[j].y > theta ? 2u : 0u) | (f[j].z > theta ? 4u : 0u) | (f[j].w > theta ? 8u : 0u);
+        if (j >= nfull) nib &= (1u << max(valid(j), 0)) - 1u;
+        mask |= nib << (4 * j);
     }
     const int mine = __reduce_add_sync(kFull, __popc(mask));
     int total = mine, base = 0;                  // survivors of the row; those ahead of this warp's run
@@ -769,7 +867,7 @@ __global__ void __launch_bounds__(WPR < 4 ? 128 : WPR * 32) stat_topk_reg_kernel
         float* yrow = p.y_dense + row * p.ld + begin;
 #pragma unroll
         for (int j = 0; j < kRegVec; ++j) {
-            const int v = v0 + 32 * j, nv = valid(j);
+            const int v = v0 + 32 * j, nv = j < nfull ? 4 : valid(j);
             const unsigned b = mask >> (4 * j);
             const float4 o = make_float4(b & 1u ? f[j].x - shift : fillv, b & 2u ? f[j].y - shift : fillv, b & 4u ? f[j].z - shift : fillv, b & 8u ? f[j].w - shift : fillv);
             if (nv == 4) {
@@ -856,14 +954,21 @@ static int topk_launch(spark_ctx* ctx, const float* x, int64_t rows, int64_t n, 
     p.theta_in = theta_in; p.moments_out = moments_out;
     p.hdr = ctx->hdr;
 
-    static const int regmode = getenv("REGMODE") ? atoi(getenv("REGMODE")) : 1;
-    if (n <= 65536 && (regmode == 1 ? (n <= 16384 || rows <= 1000000) : regmode == 2 ? n <= 16384 : false)) {
-        const int rcl = n <= 16384 ? 1 : (n <= 32768 ? 2 : 4);
+    // Lists by staging windows cost with the survivors, by ballots with the values: 2000 x 40000 at 2 / 8 / 25 % 134 / 178 / 408 us
+    // against 207 / 236 / 246.
+    p.direct = k * 10 > n ? 1 : 0;
+    // Rows in registers: up to 8192 values always (4096 x 8192, statistics 37 against 50 us, dense 49 against 71), to 16384 for lists
+    // (1000 x 16000 lists 46 against 50 us, but statistics 31 against 28); beyond that for the lists of so few rows that every block
+    // of their clusters has an SM to itself (32 x 28289 at 25 %: 10 against 16 us; 115 x 49138: 37 against 21).
+    const bool lists = idx != nullptr || val != nullptr;
+    const int64_t rcl = n <= 16384 ? 1 : (n <= 32768 ? 2 : 4);
+    if (n <= 8192 || (lists && (n <= 16384 || (n <= 65536 && 2 * rows * rcl <= ctx->num_sms)))) {
         p.chunk = ((n + rcl - 1) / rcl + 3) / 4 * 4;
+        const int cl_reg = static_cast<int>(rcl);
         const int warps = static_cast<int>((p.chunk + 4 * kRegWarpVec - 1) / (4 * kRegWarpVec));
         cudaStream_t st = static_cast<cudaStream_t>(stream);
-        const cudaError_t er = warps <= 1 ? reg_launch<1>(p, rcl, st) : warps <= 2 ? reg_launch<2>(p, rcl, st) : warps <= 4 ? reg_launch<4>(p, rcl, st)
-                             : warps <= 8 ? reg_launch<8>(p, rcl, st) : reg_launch<16>(p, rcl, st);
+        const cudaError_t er = warps <= 1 ? reg_launch<1>(p, cl_reg, st) : warps <= 2 ? reg_launch<2>(p, cl_reg, st) : warps <= 4 ? reg_launch<4>(p, cl_reg, st)
+                             : warps <= 8 ? reg_launch<8>(p, cl_reg, st) : reg_launch<16>(p, cl_reg, st);
         return er == cudaSuccess ? SPARK_OK : SPARK_ERR_CUDA;
     }
 
@@ -877,13 +982,15 @@ static int topk_launch(spark_ctx* ctx, const float* x, int64_t rows, int64_t n, 
     if (n > 16384 && (n + 3) / 4 <= kRowMaxVec && theta_in == nullptr && moments_out == nullptr) {      // the whole row fits one block: no cluster needed
         static bool row_attr_done[64] = {};
         if (ctx->device >= 0 && ctx->device < 64 && !row_attr_done[ctx->device]) {
-            if (cudaFuncSetAttribute(stat_topk_row_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kRowSmemBytes) != cudaSuccess)
+            if (cudaFuncSetAttribute(stat_topk_row_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, kRowSmemBytes) != cudaSuccess ||
+                cudaFuncSetAttribute(stat_topk_row_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, kRowSmemBytes) != cudaSuccess)
                 return SPARK_ERR_CUDA;
             row_attr_done[ctx->device] = true;
         }
         const size_t smem = kRowSmemBytes;
         const int64_t grid = rows < ctx->num_sms ? rows : ctx->num_sms;
-        stat_topk_row_kernel<<<static_cast<unsigned>(grid), kRowThreads, smem, static_cast<cudaStream_t>(stream)>>>(p);
+        if (lists) stat_topk_row_kernel<true><<<static_cast<unsigned>(grid), kRowThreads, smem, static_cast<cudaStream_t>(stream)>>>(p);
+        else stat_topk_row_kernel<false><<<static_cast<unsigned>(grid), kRowThreads, smem, static_cast<cudaStream_t>(stream)>>>(p);
         return cudaGetLastError() == cudaSuccess ? SPARK_OK : SPARK_ERR_CUDA;
     }
 
