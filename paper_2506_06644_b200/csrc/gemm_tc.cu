@@ -55,9 +55,9 @@ __global__ void __launch_bounds__(256) gemm_tc_prep_kernel(const GemmParams p) {
             }
         } else if (p.sp.split == 0 && p.sp.per == 0) {
             for (int g = 1 + blockIdx.x; g < p.sp.grid; g += gridDim.x) {
-                const int pos = stream_begin(p.sp, g), tile = pos / p.sp.call, start = tile * p.sp.call;
-                if (pos == start || stream_begin(p.sp, g - 1) > start) continue;      // between two tiles, or not the tile's first cut
-                const int row = tile * kStreamRows + (tid & 127);
+                const StreamPart part = stream_part(p.sp, g), ahead = stream_part(p.sp, g - 1);
+                if (part.c == 0 || (ahead.tile == part.tile && ahead.c > 0)) continue;      // between two tiles, or not the tile's first cut
+                const int row = part.tile * kStreamRows + (tid & 127);
                 if (row < p.n_out)
                     for (int b = tid >> 7; b < p.B; b += 2) {
                         const int64_t at = static_cast<int64_t>(b) * p.n_out + row;

@@ -68,6 +68,10 @@ span_gemm_kernel(const SpanGemm p, const __grid_constant__ CUtensorMap map_w, co
     extern __shared__ unsigned char tc_raw[];
     __shared__ SpanShared sh;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    if (tid == 64) {
+        tma_prefetch_desc(&map_w);
+        tma_prefetch_desc(&map_x);
+    }
     if (tid == 0) {
         for (int s = 0; s < kSpanStages; ++s) {
             mbar_init(smem_addr(&sh.full[s]), 1u);

@@ -103,6 +103,8 @@ span_attn_sums_kernel(const __grid_constant__ VParams p, const __grid_constant__
     extern __shared__ unsigned char tc_raw[];
     __shared__ SumShared sh;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    if (tid == 64)
+        for (const CUtensorMap* m : {&map_k1, &map_qhi, &map_qlo}) tma_prefetch_desc(m);
     if (tid == 0) {
         for (int s = 0; s < kSumSlots; ++s) {
             mbar_init(smem_addr(&sh.full[s]), 1u);
@@ -302,6 +304,8 @@ span_attn_main_kernel(const __grid_constant__ VParams p, const __grid_constant__
     extern __shared__ unsigned char tc_raw[];
     __shared__ MainShared sh;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    if (tid == 64)
+        for (const CUtensorMap* m : {&map_k1, &map_k2, &map_v, &map_qhi, &map_qlo, &map_q2hi, &map_q2lo}) tma_prefetch_desc(m);
     if (tid == 0) {
         for (int s = 0; s < kMainSlots; ++s) {
             mbar_init(smem_addr(&sh.full[s]), 1u);

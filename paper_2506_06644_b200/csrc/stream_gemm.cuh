@@ -32,6 +32,7 @@ struct StreamPlan {
     int grid, per;           // blocks; chunks a block takes (0: equal parts of the sequence or of each tile)
     int part, rem;           // an equal part is `part` chunks, one more for the first `rem` of them (of the sequence, or of a tile)
     int split;               // every tile is cut into this many pieces (0: no such regular cut)
+    uint32_t inv_split;      // 65536 / split + 1: block / split for fewer than 65536 / split blocks
     int call;                // K chunks of a tile
     int ntok;                // tokens rounded up to a multiple of 16: half of the MMAs' N; X has rows term * ntok + token
     int stages;
@@ -39,14 +40,19 @@ struct StreamPlan {
     uint32_t tmem_cols;
 };
 
-// Start of a block's part of the sequence (no 64-bit division: it sits in front of the first load).
-__host__ __device__ inline int stream_begin(const StreamPlan& sp, int block) {
-    if (sp.per > 0) return block < sp.grid ? block * sp.per : sp.total;
+// A block's part of the sequence: its first tile, the K chunk it starts at and the number of chunks.  No division where every
+// block has one piece of a tile: this sits in front of the first load.
+struct StreamPart {
+    int tile, c, n;
+};
+__host__ __device__ inline StreamPart stream_part(const StreamPlan& sp, int block) {
     if (sp.split > 0) {
-        const int tile = block / sp.split, i = block - tile * sp.split;
-        return tile * sp.call + i * sp.part + (i < sp.rem ? i : sp.rem);
+        const int tile = static_cast<int>(static_cast<uint32_t>(block) * sp.inv_split >> 16), i = block - tile * sp.split;
+        return StreamPart{tile, i * sp.part + (i < sp.rem ? i : sp.rem), sp.part + (i < sp.rem ? 1 : 0)};
     }
-    return block * sp.part + (block < sp.rem ? block : sp.rem);
+    const int p0 = sp.per > 0 ? block * sp.per : block * sp.part + (block < sp.rem ? block : sp.rem), tile = p0 / sp.call;
+    const int left = sp.total - p0, n = sp.per > 0 ? (left < sp.per ? left : sp.per) : sp.part + (block < sp.rem ? 1 : 0);
+    return StreamPart{tile, p0 - tile * sp.call, n};
 }
 
 // Host: fills in the plan for at most `smem_limit` bytes of dynamic shared memory.  False: does not fit.
@@ -70,6 +76,7 @@ inline bool stream_plan(StreamPlan& sp, int sms, int tiles, int call, int tokens
     const int of = sp.split > 0 ? call : sp.total, by = sp.split > 0 ? sp.split : sp.grid;
     sp.part = of / by;
     sp.rem = of % by;
+    sp.inv_split = sp.split > 0 ? 65536u / static_cast<uint32_t>(sp.split) + 1u : 0u;
     sp.ntok = (tokens + 15) & ~15;
     sp.stage_bytes = kStreamTileBytes + 2 * sp.ntok * kChunk * 2;
     const int fit = static_cast<int>((smem_limit - 1024) / sp.stage_bytes);
@@ -89,19 +96,24 @@ template <class Epi>
 __device__ __forceinline__ void stream_gemm(const StreamPlan& sp, StreamShared& sh, unsigned char* raw, const CUtensorMap* map_w,
                                             const CUtensorMap* map_x, WsHeader* hdr, Epi epi) {
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    const int p0 = stream_begin(sp, blockIdx.x), p1 = stream_begin(sp, blockIdx.x + 1), n = p1 - p0;
+    const StreamPart part = stream_part(sp, blockIdx.x);
+    const int n = part.n;
     const uint32_t xbytes = static_cast<uint32_t>(2 * sp.ntok) * (kChunk * 2);
     const int stages = sp.stages;
-    if (tid == 0) {
-        for (int s = 0; s < stages; ++s) {
-            mbar_init(smem_addr(&sh.full[s]), 1u);
-            mbar_init(smem_addr(&sh.empty[s]), 1u);
-        }
-        for (int b = 0; b < 2; ++b) {
+    if (tid == 64) {         // descriptors first: a miss behind the dependency wait costs 0.3 us
+        tma_prefetch_desc(map_w);
+        tma_prefetch_desc(map_x);
+    }
+    if (tid < 32) {
+        if (tid < stages) {
+            mbar_init(smem_addr(&sh.full[tid]), 1u);
+            mbar_init(smem_addr(&sh.empty[tid]), 1u);
+        } else if (tid < stages + 2) {
+            const int b = tid - stages;
             mbar_init(smem_addr(&sh.acc_full[b]), 1u);
             mbar_init(smem_addr(&sh.acc_empty[b]), 4u);
         }
-        sh.abort_flag = 0;
+        if (tid == 0) sh.abort_flag = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
     }
@@ -116,7 +128,7 @@ __device__ __forceinline__ void stream_gemm(const StreamPlan& sp, StreamShared& 
 
     if (warp == 0) {
         if (lane == 0) {
-            int tile = p0 / sp.call, c = p0 - tile * sp.call, cx = c;
+            int tile = part.tile, c = part.c, cx = c;
             const int pre = min(n, stages);
             for (int i = 0; i < pre; ++i) {
                 const uint32_t bar = smem_addr(&sh.full[i]);
@@ -152,15 +164,16 @@ __device__ __forceinline__ void stream_gemm(const StreamPlan& sp, StreamShared& 
     } else if (warp == 1) {
         // the whole warp walks the loop; one elected lane issues
         const uint32_t elected = elect_lane(), idesc = instr_desc(128, 2 * sp.ntok, false);
-        int s = 0, pos = p0, seg = 0;
+        int s = 0, seg = 0;
         uint32_t parity = 0u;
         bool ok = true;
-        while (pos < p1 && ok) {
-            const int end = min(p1, (pos / sp.call + 1) * sp.call), b = seg & 1;
+        for (int done = 0, len = min(n, sp.call - part.c); done < n && ok; done += len, len = min(n - done, sp.call)) {
+            const int b = seg & 1;
             if (seg >= 2) ok = __all_sync(kFull, mbar_wait(smem_addr(&sh.acc_empty[b]), ((seg >> 1) & 1) ^ 1, abort_flag));
             const uint32_t acc = tmem + static_cast<uint32_t>(b * 2 * sp.ntok);
             tc_fence_after();
-            for (uint32_t more = 0u; pos < end && ok; ++pos, more = 1u) {
+            uint32_t more = 0u;
+            for (int i = 0; i < len; ++i, more = 1u) {
                 ok = __all_sync(kFull, mbar_wait(smem_addr(&sh.full[s]), parity, abort_flag));
                 if (!ok) break;
                 tc_fence_after();
@@ -178,21 +191,20 @@ __device__ __forceinline__ void stream_gemm(const StreamPlan& sp, StreamShared& 
     } else {
         const int q = warp & 3;                                    // tensor-memory lanes 32 q .. 32 q + 31
         dep_wait();
-        int pos = p0, seg = 0;
-        while (pos < p1) {
-            const int tile = pos / sp.call, end = min(p1, (tile + 1) * sp.call), b = seg & 1;
+        int seg = 0, tile = part.tile;
+        for (int done = 0, len = min(n, sp.call - part.c); done < n; done += len, len = min(n - done, sp.call), ++tile) {
+            const int b = seg & 1;
             if (!__all_sync(kFull, mbar_wait(smem_addr(&sh.acc_full[b]), (seg >> 1) & 1, abort_flag))) break;      // warp-uniform: tcgen05.ld is warp-wide
             tc_fence_after();
             const uint32_t taddr = tmem + static_cast<uint32_t>(b * 2 * sp.ntok) + (static_cast<uint32_t>(q * 32) << 16);
             for (int n0 = 0; n0 < sp.ntok; n0 += 16) {
                 float v[16];
                 tmem_ld16_sum(taddr + n0, taddr + sp.ntok + n0, v);
-                epi(tile, end - pos == sp.call, q * 32 + lane, n0, v);
+                epi(tile, len == sp.call, q * 32 + lane, n0, v);
             }
             tc_fence_before();
             __syncwarp();
             if (lane == 0) asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_addr(&sh.acc_empty[b])) : "memory");
-            pos = end;
             ++seg;
         }
     }
