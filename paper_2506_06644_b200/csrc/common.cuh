@@ -318,6 +318,13 @@ __device__ __forceinline__ float gelu_tanh(float a) {
     const float c = 0.7978845608028654f;   // sqrt(2/pi)
     return 0.5f * a * (1.0f + tanhf(c * (a + 0.044715f * a * a * a)));
 }
+// The tanh form of GELU as a x sigmoid(2 sqrt(2/pi) (a + 0.044715 a^3)): the same function with one exponential and one division.
+__device__ __forceinline__ float gelu_logistic(float a) {
+    const float y = a * fmaf(0.1029432397f, a * a, 2.302208198f);      // 2 sqrt(2/pi) log2(e) (1, 0.044715)
+    float e;
+    asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(e) : "f"(-y));
+    return __fdividef(a, 1.f + e);
+}
 __device__ __forceinline__ float gelu_erf(float a) {
     return 0.5f * a * (1.0f + erff(a * 0.7071067811865476f));
 }

@@ -53,14 +53,6 @@ struct SpanShared {
     int abort_flag;
 };
 
-// The tanh form of GELU as a x sigmoid(2 sqrt(2/pi) (a + 0.044715 a^3)): the same function with one exponential and one division.
-__device__ __forceinline__ float gelu_logistic(float a) {
-    const float y = a * fmaf(0.1029432397f, a * a, 2.302208198f);      // 2 sqrt(2/pi) log2(e) (1, 0.044715)
-    float e;
-    asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(e) : "f"(-y));
-    return __fdividef(a, 1.f + e);
-}
-
 // MN: the matrix is stored [K][rows] (V); U: the epilogue forms the activations.
 template <bool MN, bool U>
 __global__ void __launch_bounds__(kSpanThreads, 1)

@@ -1,7 +1,6 @@
 // Pieces shared by the kernels that run on the fifth-generation tensor cores (tcgen05): PTX wrappers for
 // mbarriers, TMA tile loads, tensor-memory allocation, MMA issue and accumulator reads; the operand and
-// instruction descriptors; the block-level set-up / tear-down of a TMA -> MMA -> epilogue pipeline with
-// bounded waits; and the host-side construction of tensor maps.  Every wait is bounded: a role whose wait
+// instruction descriptors; and the host-side construction of tensor maps.  Every wait is bounded: a role whose wait
 // runs out raises the block's abort flag, which ends the other roles' waits; the block then lets its copies
 // in flight land (bounded), frees its tensor memory and records SPARK_ERR_TIMEOUT.
 #pragma once
@@ -146,59 +145,6 @@ __device__ __forceinline__ unsigned pack2_bf16(float lo, float hi) {
     unsigned r;
     asm("cvt.rn.bf16x2.f32 %0, %1, %2;" : "=r"(r) : "f"(hi), "f"(lo));
     return r;
-}
-
-// ---- block-level pieces shared by the two tensor-core kernels ------------------------------------------
-struct TcShared {
-    unsigned long long full[8];     // stage filled (TMA transaction bytes)
-    unsigned long long empty[8];    // stage drained (tcgen05.commit)
-    unsigned long long accum;       // accumulators final
-    uint32_t tmem;                  // tensor-memory base address written by tcgen05.alloc
-    int abort_flag;                 // a bounded wait of some role ran out
-    double colsum[4][64][2];        // per epilogue warp and token: partial sums (kernels that reduce over rows)
-};
-
-template <int STAGES>
-__device__ __forceinline__ uint32_t tc_setup(TcShared& sh, unsigned char* raw, uint32_t tmem_cols) {
-    const int tid = threadIdx.x, warp = tid >> 5;
-    if (tid == 0) {
-        for (int s = 0; s < STAGES; ++s) {
-            mbar_init(smem_addr(&sh.full[s]), 1u);
-            mbar_init(smem_addr(&sh.empty[s]), 1u);
-        }
-        mbar_init(smem_addr(&sh.accum), 1u);
-        sh.abort_flag = 0;
-        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-    }
-    if (warp == 1) tmem_alloc(smem_addr(&sh.tmem), tmem_cols);
-    tc_fence_before();
-    __syncthreads();
-    tc_fence_after();
-    return (smem_addr(raw) + 1023u) & ~1023u;         // operand tiles need 1024-byte alignment (swizzle atom)
-}
-
-// After a wait ran out: the producer thread gives its copies in flight a bounded time to land, so
-// that none writes into the shared memory of a block that has gone.
-template <int STAGES>
-__device__ __forceinline__ void tc_drain(TcShared& sh, int issued) {
-    for (int i = max(0, issued - STAGES); i < issued; ++i) {
-        const uint32_t bar = smem_addr(&sh.full[i % STAGES]), parity = static_cast<uint32_t>(i / STAGES) & 1u;
-        const long long t0 = clock64();
-        while (!mbar_try(bar, parity))
-            if (clock64() - t0 > kTcSpinLimit) break;
-    }
-}
-
-__device__ __forceinline__ void tc_finish(TcShared& sh, uint32_t tmem_cols, WsHeader* hdr) {
-    tc_fence_before();
-    __syncthreads();
-    if ((threadIdx.x >> 5) == 1) {
-        __syncwarp();
-        tc_fence_after();
-        tmem_free(sh.tmem, tmem_cols);
-    }
-    if (threadIdx.x == 0 && sh.abort_flag != 0) atomicCAS(&hdr->status, SPARK_OK, SPARK_ERR_TIMEOUT);
 }
 
 // ---- host side ---------------------------------------------------------------------------------------------
