@@ -47,6 +47,10 @@ int ffn_mma_launch(spark_ctx* ctx, FfnParams& p, cudaStream_t stream);
 int ffn_tc_launch(spark_ctx* ctx, FfnParams& p, cudaStream_t stream);
 size_t ffn_tc_workspace_bytes(int64_t d, int64_t d_ff);
 
+// The same for 5..16 tokens of a small model, called by ffn_tc_launch() (ffn_chain.cu).
+int ffn_chain_launch(spark_ctx* ctx, FfnParams& p, cudaStream_t stream);
+size_t ffn_chain_workspace_bytes(int64_t d, int64_t d_ff);
+
 // 2..4 tokens without tensor cores (ffn_few.cu); SPARK_ERR_WORKSPACE = shape not served.
 int ffn_few_launch(spark_ctx* ctx, FfnParams& p, int wdtype, cudaStream_t stream);
 

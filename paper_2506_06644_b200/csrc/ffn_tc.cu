@@ -496,7 +496,10 @@ ffn_tc_kernel(const TcParams p, const __grid_constant__ CUtensorMap map_k1, cons
 
 namespace spark {
 
-size_t ffn_tc_workspace_bytes(int64_t d, int64_t d_ff) { return tc_region_bytes(d, d_ff); }
+size_t ffn_tc_workspace_bytes(int64_t d, int64_t d_ff) {
+    const size_t one = tc_region_bytes(d, d_ff), chain = ffn_chain_workspace_bytes(d, d_ff);
+    return one > chain ? one : chain;
+}
 
 // SPARK_ERR_WORKSPACE = shape or workspace not served by this path (the caller falls back).
 int ffn_tc_launch(spark_ctx* ctx, FfnParams& f, cudaStream_t stream) {
@@ -506,6 +509,12 @@ int ffn_tc_launch(spark_ctx* ctx, FfnParams& f, cudaStream_t stream) {
     if (ctx->scratch == nullptr || ctx->scratch_bytes < kAttnCellBytes + tc_region_bytes(d, d_ff)) return SPARK_ERR_WORKSPACE;
     if ((reinterpret_cast<uintptr_t>(f.K1t) | reinterpret_cast<uintptr_t>(f.K2t) | reinterpret_cast<uintptr_t>(f.Vt)) & 15u) return SPARK_ERR_WORKSPACE;
 
+    // Up to 16 MB of weights (2.5 us of the stream) and 16 tokens as a chain of kernels: a barrier costs more than a chained launch, a
+    // launch stops the stream.  Measured at 1 MB, 6 MB: 16.3, 16.4 us here and 14.4, 14.4 there; at 67 MB, 6 tokens: 26.1 and 26.6.
+    if (B <= 16 && static_cast<int64_t>(d) * d_ff * 4 <= (16 << 20)) {
+        const int rc = ffn_chain_launch(ctx, f, stream);
+        if (rc != SPARK_ERR_WORKSPACE) return rc;
+    }
     TcParams p;
     p.f = f;
     p.g = tc_region(ctx->scratch + kAttnCellBytes, d);             // behind the attention's persistent cells
@@ -523,7 +532,9 @@ int ffn_tc_launch(spark_ctx* ctx, FfnParams& f, cudaStream_t stream) {
     p.stage_bytes = kStreamTileBytes + 2 * p.ntok * kChunk * 2;
     const int limit = ctx->max_smem_optin - static_cast<int>(sizeof(FfnShared)) - 256, fit = (limit - 1024) / p.stage_bytes;
     if (fit < 2) return SPARK_ERR_WORKSPACE;
+    const int most = per * ((r + kChunk - 1) / kChunk + (d - r + kChunk - 1) / kChunk) + (cvn + p.ksplit - 1) / p.ksplit;      // chunks of a block
     p.stages = fit < kMaxStages ? fit : kMaxStages;
+    if (p.stages > most) p.stages = most;              // small shapes: room for the blocks of the kernel ahead
     p.tmem_cols = 32;
     while (p.tmem_cols < static_cast<uint32_t>(4 * per * p.ntok)) p.tmem_cols *= 2;
 
@@ -532,9 +543,9 @@ int ffn_tc_launch(spark_ctx* ctx, FfnParams& f, cudaStream_t stream) {
         !make_map(&m_x1, p.g.xs, 2 * p.ntok, r, d, 2 * p.ntok, false) || !make_map(&m_x2, p.g.xs + r, 2 * p.ntok, d - r, d, 2 * p.ntok, false) ||
         !make_map(&m_v, f.Vt, d_ff, d, d, kChunk, true) || !make_map(&m_u, p.g.us, 2 * p.ntok, d_ff, d_ff, 2 * p.ntok, false))
         return SPARK_ERR_WORKSPACE;
-    // More than half of an SM's shared memory, always: blocks that hold tensor memory and wait for other blocks never share an SM with
-    // blocks of another such kernel, which might hold the columns that they wait for.
-    const size_t want = static_cast<size_t>(p.stages) * p.stage_bytes + 1024, least = 120 * 1024;
+    // At least the share of an SM's shared memory that its columns are of tensor memory: blocks that hold columns while they wait for
+    // other blocks then never share an SM with so many of their kind that one waits for columns.
+    const size_t want = static_cast<size_t>(p.stages) * p.stage_bytes + 1024, least = (static_cast<size_t>(ctx->max_smem_optin) + 1024) * p.tmem_cols / 512;
     const void* kern = reinterpret_cast<const void*>(ffn_tc_kernel);
     if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, limit) != cudaSuccess) return SPARK_ERR_CUDA;
     void* args[] = {&p, &m_k1, &m_x1, &m_k2, &m_x2, &m_v, &m_u};

@@ -110,7 +110,7 @@ __global__ void __launch_bounds__(kTcThreads, 1)
 gemm_tc_kernel(const GemmParams p, const __grid_constant__ CUtensorMap map_w, const __grid_constant__ CUtensorMap map_x) {
     extern __shared__ unsigned char tc_raw[];
     __shared__ StreamShared sh;
-    stream_gemm(p.sp, sh, tc_raw, &map_w, &map_x, p.hdr, [&](int tile, bool whole, int r, int n0, const float (&v)[16]) {
+    stream_gemm<0>(p.sp, sh, tc_raw, &map_w, &map_x, p.hdr, [] {}, [&](int tile, bool whole, int r, int n0, const float (&v)[16]) {
         const int row = tile * kStreamRows + r;
         if (row >= p.n_out) return;
         const int64_t at = static_cast<int64_t>(n0) * p.n_out + row;

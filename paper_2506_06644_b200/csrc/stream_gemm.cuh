@@ -34,6 +34,7 @@ struct StreamPlan {
     int split;               // every tile is cut into this many pieces (0: no such regular cut)
     uint32_t inv_split;      // 65536 / split + 1: block / split for fewer than 65536 / split blocks
     int call;                // K chunks of a tile
+    int rows;                // rows of a tile: 128, or a smaller multiple of 8 (the MMAs' other rows read whatever lies behind and are dropped)
     int ntok;                // tokens rounded up to a multiple of 16: half of the MMAs' N; X has rows term * ntok + token
     int stages;
     int stage_bytes;
@@ -55,16 +56,24 @@ __host__ __device__ inline StreamPart stream_part(const StreamPlan& sp, int bloc
     return StreamPart{tile, p0 - tile * sp.call, n};
 }
 
-// Host: fills in the plan for at most `smem_limit` bytes of dynamic shared memory.  False: does not fit.
-inline bool stream_plan(StreamPlan& sp, int sms, int tiles, int call, int tokens, size_t smem_limit) {
+// Alignment of the first tile, and room behind the last one for an operand of 128 rows that starts in it.
+inline size_t stream_slack(const StreamPlan& sp) { return 1024 + static_cast<size_t>(sp.stage_bytes < kStreamTileBytes ? kStreamTileBytes - sp.stage_bytes : 0); }
+
+// Host: fills in the plan for at most `smem_limit` bytes of dynamic shared memory.  whole: a block takes one whole tile, however many
+// there are (the caller needs whole products).  False: does not fit.
+inline bool stream_plan(StreamPlan& sp, int sms, int tiles, int call, int tokens, size_t smem_limit, bool whole = false, int rows = kStreamRows) {
     sp.call = call;
     sp.total = tiles * call;
+    sp.rows = rows;
     sp.per = sp.split = 0;
     // A piece of a tile costs its block an epilogue (1.5 to 4 us with the reductions of 16 to 64 tokens), so blocks get one piece
     // of one tile, or whole tiles, where that leaves 0.6 / 0.9 of the SMs busy: fewer SMs still draw what HBM gives (4096 x 2304,
     // 64 tokens: 128 blocks of one piece 9.7 us, 148 equal parts of two pieces each 15.4 us).  Otherwise equal parts.
     const int ks = sms / tiles < call ? sms / tiles : call, m = (tiles + sms - 1) / sms;
-    if (ks >= 1 && (tiles * ks * 10 >= sms * 6 || ks == call)) {
+    if (whole) {
+        sp.per = call;
+        sp.grid = tiles;
+    } else if (ks >= 1 && (tiles * ks * 10 >= sms * 6 || ks == call)) {
         sp.split = ks;
         sp.grid = tiles * ks;
     } else if (tiles > sms && m <= 4 && (tiles + m - 1) / m * 10 >= sms * 9) {
@@ -78,27 +87,41 @@ inline bool stream_plan(StreamPlan& sp, int sms, int tiles, int call, int tokens
     sp.rem = of % by;
     sp.inv_split = sp.split > 0 ? 65536u / static_cast<uint32_t>(sp.split) + 1u : 0u;
     sp.ntok = (tokens + 15) & ~15;
-    sp.stage_bytes = kStreamTileBytes + 2 * sp.ntok * kChunk * 2;
-    const int fit = static_cast<int>((smem_limit - 1024) / sp.stage_bytes);
+    sp.stage_bytes = (rows + 2 * sp.ntok) * kChunk * 2;
+    const int fit = static_cast<int>((smem_limit - stream_slack(sp)) / sp.stage_bytes);
     // more than eight stages (128 KB of weights in flight per SM, three times what the latency of HBM needs) only delays the
     // small loads of the kernel ahead that queue behind them
     sp.stages = fit < kStreamMaxStages ? fit : kStreamMaxStages;
+    // no more than a block has chunks, and a second accumulator only for a second piece: blocks of small products fit on an SM beside
+    // those of the kernel ahead and set up under its tail
+    const int most = sp.per > 0 ? sp.per : sp.part + (sp.rem > 0 ? 1 : 0);
+    if (sp.stages > most) sp.stages = most > 2 ? most : 2;
     uint32_t cols = 32;
-    while (cols < static_cast<uint32_t>(4 * sp.ntok)) cols *= 2;
+    while (cols < static_cast<uint32_t>((sp.split > 0 || sp.per == call ? 2 : 4) * sp.ntok)) cols *= 2;
     sp.tmem_cols = cols;
     return sp.stages >= 2 && cols <= 512 && tiles > 0 && call > 0;
 }
-inline size_t stream_smem(const StreamPlan& sp) { return static_cast<size_t>(sp.stages) * sp.stage_bytes + 1024; }
+inline size_t stream_smem(const StreamPlan& sp) { return static_cast<size_t>(sp.stages) * sp.stage_bytes + stream_slack(sp); }
 
-// One block's work.  epi(tile, whole, row, n0, v): sixteen tokens' values of one row (0..127) of a tile; `whole`: the block holds
-// all of the tile's K range.
-template <class Epi>
+// Variants of stream_gemm():
+//   kStreamEarlyX   X is complete when the kernel starts: its producer is two places ahead in the stream and the kernel ahead is
+//                   kStreamLate.  The products run before griddepcontrol.wait; only the epilogue needs the kernel ahead.
+//   kStreamLate     the kernel behind may start once this one has seen the end of the kernel ahead (implied by kStreamEarlyX);
+//                   otherwise at once: it only requests its weights before it waits for this kernel
+//   kStreamMN       A is stored [K][rows] (two boxes of 64 rows per K chunk)
+constexpr int kStreamEarlyX = 1, kStreamLate = 2, kStreamMN = 4;
+
+// One block's work.  before() runs in the four epilogue warps once the kernel ahead is complete.  epi(tile, whole, row, n0, v):
+// sixteen tokens' values of one row of a tile (a whole warp calls it; rows from sp.rows on are to be dropped); `whole`: the block
+// holds all of the tile's K range.
+template <int V, class Before, class Epi>
 __device__ __forceinline__ void stream_gemm(const StreamPlan& sp, StreamShared& sh, unsigned char* raw, const CUtensorMap* map_w,
-                                            const CUtensorMap* map_x, WsHeader* hdr, Epi epi) {
+                                            const CUtensorMap* map_x, WsHeader* hdr, Before before, Epi epi) {
+    constexpr bool kEarlyX = (V & kStreamEarlyX) != 0, kLate = (V & (kStreamEarlyX | kStreamLate)) != 0, kMN = (V & kStreamMN) != 0;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const StreamPart part = stream_part(sp, blockIdx.x);
     const int n = part.n;
-    const uint32_t xbytes = static_cast<uint32_t>(2 * sp.ntok) * (kChunk * 2);
+    const uint32_t wbytes = static_cast<uint32_t>(sp.rows) * (kChunk * 2), stage_bytes = static_cast<uint32_t>(sp.stage_bytes);
     const int stages = sp.stages;
     if (tid == 64) {         // descriptors first: a miss behind the dependency wait costs 0.3 us
         tma_prefetch_desc(map_w);
@@ -124,7 +147,15 @@ __device__ __forceinline__ void stream_gemm(const StreamPlan& sp, StreamShared& 
     const uint32_t base = (smem_addr(raw) + 1023u) & ~1023u;
     const uint32_t tmem = sh.tmem;
     volatile int* abort_flag = &sh.abort_flag;
-    dep_trigger();           // the kernel behind only requests its weights before it waits for this one
+    if (!kLate) dep_trigger();
+    auto load_w = [&](uint32_t dst, uint32_t bar, int c, int tile) {
+        if (kMN) {
+            tma_load_2d(dst, map_w, bar, tile * kStreamRows, c * kChunk);
+            tma_load_2d(dst + kChunk * 128, map_w, bar, tile * kStreamRows + 64, c * kChunk);
+        } else {
+            tma_load_2d(dst, map_w, bar, c * kChunk, tile * sp.rows);
+        }
+    };
 
     if (warp == 0) {
         if (lane == 0) {
@@ -132,23 +163,23 @@ __device__ __forceinline__ void stream_gemm(const StreamPlan& sp, StreamShared& 
             const int pre = min(n, stages);
             for (int i = 0; i < pre; ++i) {
                 const uint32_t bar = smem_addr(&sh.full[i]);
-                mbar_expect_tx(bar, kStreamTileBytes + xbytes);
-                tma_load_2d(base + i * sp.stage_bytes, map_w, bar, c * kChunk, tile * kStreamRows);
+                mbar_expect_tx(bar, stage_bytes);
+                load_w(base + i * stage_bytes, bar, c, tile);
                 if (++c == sp.call) { c = 0; ++tile; }
             }
-            dep_wait();
+            if (!kEarlyX) dep_wait();
             for (int i = 0; i < pre; ++i) {
-                tma_load_2d(base + i * sp.stage_bytes + kStreamTileBytes, map_x, smem_addr(&sh.full[i]), cx * kChunk, 0);
+                tma_load_2d(base + i * stage_bytes + wbytes, map_x, smem_addr(&sh.full[i]), cx * kChunk, 0);
                 if (++cx == sp.call) cx = 0;
             }
             int s = 0, issued = pre;
             uint32_t parity = 0u;
             for (int i = pre; i < n; ++i) {
                 if (!mbar_wait(smem_addr(&sh.empty[s]), parity, abort_flag)) break;
-                const uint32_t bar = smem_addr(&sh.full[s]), dst = base + s * sp.stage_bytes;
-                mbar_expect_tx(bar, kStreamTileBytes + xbytes);
-                tma_load_2d(dst, map_w, bar, c * kChunk, tile * kStreamRows);
-                tma_load_2d(dst + kStreamTileBytes, map_x, bar, c * kChunk, 0);
+                const uint32_t bar = smem_addr(&sh.full[s]), dst = base + s * stage_bytes;
+                mbar_expect_tx(bar, stage_bytes);
+                load_w(dst, bar, c, tile);
+                tma_load_2d(dst + wbytes, map_x, bar, c * kChunk, 0);
                 if (++c == sp.call) { c = 0; ++tile; }
                 if (++s == stages) { s = 0; parity ^= 1u; }
                 issued = i + 1;
@@ -163,7 +194,7 @@ __device__ __forceinline__ void stream_gemm(const StreamPlan& sp, StreamShared& 
         }
     } else if (warp == 1) {
         // the whole warp walks the loop; one elected lane issues
-        const uint32_t elected = elect_lane(), idesc = instr_desc(128, 2 * sp.ntok, false);
+        const uint32_t elected = elect_lane(), idesc = instr_desc(128, 2 * sp.ntok, kMN);
         int s = 0, seg = 0;
         uint32_t parity = 0u;
         bool ok = true;
@@ -177,11 +208,12 @@ __device__ __forceinline__ void stream_gemm(const StreamPlan& sp, StreamShared& 
                 ok = __all_sync(kFull, mbar_wait(smem_addr(&sh.full[s]), parity, abort_flag));
                 if (!ok) break;
                 tc_fence_after();
-                const uint32_t a0 = base + s * sp.stage_bytes;
-                const uint64_t ad = smem_desc(a0, 0u, 1024u), xd = smem_desc(a0 + kStreamTileBytes, 0u, 1024u);
+                const uint32_t a0 = base + s * stage_bytes;
+                // 16 K elements further: 32 bytes in a row of K, or sixteen rows of 128 bytes
+                const uint64_t ad = smem_desc(a0, kMN ? kChunk * 128u : 0u, 1024u), xd = smem_desc(a0 + wbytes, 0u, 1024u);
 #pragma unroll
                 for (int j = 0; j < kChunk / 16; ++j)      // descriptors count in 16-byte units
-                    umma_bf16_elected(acc, ad + 2 * j, xd + 2 * j, idesc, j == 0 ? more : 1u, elected);
+                    umma_bf16_elected(acc, ad + (kMN ? 128 : 2) * j, xd + 2 * j, idesc, j == 0 ? more : 1u, elected);
                 umma_commit_elected(smem_addr(&sh.empty[s]), elected);
                 if (++s == stages) { s = 0; parity ^= 1u; }
             }
@@ -191,13 +223,15 @@ __device__ __forceinline__ void stream_gemm(const StreamPlan& sp, StreamShared& 
     } else {
         const int q = warp & 3;                                    // tensor-memory lanes 32 q .. 32 q + 31
         dep_wait();
+        if (kLate) dep_trigger();
+        before();
         int seg = 0, tile = part.tile;
         for (int done = 0, len = min(n, sp.call - part.c); done < n; done += len, len = min(n - done, sp.call), ++tile) {
             const int b = seg & 1;
             if (!__all_sync(kFull, mbar_wait(smem_addr(&sh.acc_full[b]), (seg >> 1) & 1, abort_flag))) break;      // warp-uniform: tcgen05.ld is warp-wide
             tc_fence_after();
             const uint32_t taddr = tmem + static_cast<uint32_t>(b * 2 * sp.ntok) + (static_cast<uint32_t>(q * 32) << 16);
-            for (int n0 = 0; n0 < sp.ntok; n0 += 16) {
+            for (int n0 = 0; n0 < sp.ntok && q * 32 < sp.rows; n0 += 16) {
                 float v[16];
                 tmem_ld16_sum(taddr + n0, taddr + sp.ntok + n0, v);
                 epi(tile, len == sp.call, q * 32 + lane, n0, v);
