@@ -16,12 +16,18 @@
 //   wait    a warp per head polls that head's cells until every piece of the segment has arrived
 //           and forms theta (Eq. 11); no grid-wide barrier: only the blocks that share a segment
 //           wait for one another.
-//   pass 2  every warp selects among its own tokens (ballot), and only for those reads the k2c and
-//           vc rows: gate = softplus(k2c[t] . q[r:]), weights exp(s_t - max score) (the cells carry
+//   pass 2  every warp selects among its own tokens, the piece's survivors are shared out evenly (up to
+//           eight rows in flight per warp), and only for those it reads the k2c and vc rows: gate = softplus(k2c[t] . q[r:]), weights exp(s_t - max score) (the cells carry
 //           the head's largest score, so every piece uses the same reference), value reduction;
 //           the block adds its sum of weights and its weighted values to the head's accumulators
 //           with vector reductions; the block that completes a segment last divides.  Inside
 //           spark_layer_decode the division is left to the output projection that follows.
+//
+// What bounds it: the predictor slice's stream for long caches (eight sequences of 18432 to 32768 tokens, 2B heads:
+// 35 us of pass 1 at the copy rate), then a chain of latencies (the exchange 2 us, lists 1, gather 2.5, reductions 1 to 3).
+// Measured, pass 2 one piece after the other, a vote per 32 tokens and four rows in flight -> as it is: those eight sequences
+// 62.4 -> 56.2 us; 9B heads, FP8 cache, 3 x 16001: 28.7 -> 26.8; eight heads per KV head, 4 x 8000: 37.3 -> 30.4; one
+// sequence of 4096: 14.5 both.
 #include "kernels.h"
 
 using namespace spark;
@@ -30,7 +36,6 @@ namespace {
 
 constexpr int kThreads = 512;
 constexpr int kWarps = kThreads / kWarp;
-constexpr int kZc = 4;                // pieces per block whose quantile is cached between the passes
 constexpr int kPartPad = 8;           // floats in front of a partial accumulator: [0] max, [1] sum
 
 // FP8 predictor slice on the tensor cores (r = 128, one or two query heads per KV head): a warp takes 16 cached
@@ -90,7 +95,6 @@ struct AttnParams {
     int defer;         // 1: leave o unnormalised and the cells for the next kernel to clear
     PrefetchSpec pf;   // weights of the kernel after this one, asked into L2 once the first predictor rows are in flight
     int check_finite;  // SPARK_CHECK_FINITE: non-finite score sums are reported in the device status
-    int long_share;    // 1: a block owns 800 or more tokens of the slice
     int mma_pass;      // 1: bf16 predictor pass on the tensor cores (long shares; r = 128, at most two heads per KV head)
     int pre_stable;    // 1: the kernel directly before this one writes neither ctx_len nor cache rows other than each
                        //    sequence's newest, so lengths and older rows may be read before dep_wait()
@@ -121,18 +125,16 @@ __global__ void __launch_bounds__(kThreads, 1) attn_kernel(const AttnParams p) {
     const int NS = p.B * p.n_kv;
     const int hd = p.hd, r = p.r, d2 = hd - r;
     int* segoff = reinterpret_cast<int*>(smem_raw);                       // [NS + 1], padded
-    float* qs = reinterpret_cast<float*>(segoff + ((NS + 1 + 3) & ~3));   // [GQ][hd]
-    float* wpart = qs + GQ * hd;                                          // [kWarps][hd + kPartPad]
+    float* qs0 = reinterpret_cast<float*>(segoff + ((NS + 1 + 3) & ~3));  // [2][GQ][hd]: queries of the block's even and odd pieces
+    float* wpart = qs0 + 2 * GQ * hd;                                          // [kWarps][hd + kPartPad]
     float* sc_s = wpart + kWarps * (hd + kPartPad);                       // [GQ][ntok] when sc_smem
     int* sel_tok = reinterpret_cast<int*>(sc_s + GQ * p.ntok);            // [GQ][ntok] when sel_list: surviving tokens
     float* sel_a = reinterpret_cast<float*>(sel_tok + GQ * p.ntok);       // [GQ][ntok]              their s - s_max
-    __shared__ int sel_n[GQ];
+    __shared__ int sel_n[2][GQ];
     __shared__ double red[kWarps][GQ][2];
     __shared__ float redm[kWarps][GQ];
-    __shared__ float theta_s[GQ], smax_s[GQ];
-    __shared__ double zcache[kZc];
-    __shared__ double s_z;
-    __shared__ int s_last, s_fail, s_aligned;
+    __shared__ float theta_s[2][GQ], smax_s[2][GQ];            // of the pieces in hand
+    __shared__ int s_last[2], s_fail, s_aligned;
     __shared__ __align__(16) unsigned char q8[sizeof(K1T) == 1 ? 8 * kQ8Stride : (M16 ? 8 * kQ16Stride : 16)];   // tensor-core pass 1: query terms
     __shared__ float qsc[8];                                                             //   and their scales, per column
     __shared__ int segblk[AL ? kMaxAlignedSegs + 1 : 1];   // first block of every segment (aligned cut)
@@ -326,6 +328,7 @@ __global__ void __launch_bounds__(kThreads, 1) attn_kernel(const AttnParams p) {
             const int b = seg / p.n_kv, g = seg - b * p.n_kv;
             const int lo = seq_len(b) - L;
             const int off = static_cast<int>(f - f0) - tb;           // score slot of token t: off + t
+            float* qs = qs0 + (ord & 1) * GQ * hd;
             for (int i = tid; i < GQ * hd; i += kThreads) qs[i] = p.q[(static_cast<int64_t>(b) * p.n_q + g * GQ) * hd + i];
             if (tb == 0 && p.count != nullptr && tid < GQ) p.count[b * p.n_q + g * GQ + tid] = 0;
             if (tb == 0) {      // the segment's first piece clears the heads' accumulators before it arrives
@@ -333,9 +336,6 @@ __global__ void __launch_bounds__(kThreads, 1) attn_kernel(const AttnParams p) {
                 for (int i = tid; i < GQ * hd; i += kThreads) ob[i] = 0.f;
                 if (tid < GQ) p.lsum[b * p.n_q + g * GQ + tid] = 0.f;
             }
-            if (tid == kThreads - 1 && ord < kZc)
-                zcache[ord] = p.k_attn >= L ? 0.0
-                              : (p.zs != nullptr ? p.zs[b] : -normcdfinv(static_cast<double>(p.k_attn) / static_cast<double>(L)));
             __syncthreads();
             if constexpr (sizeof(K1T) == 1) {
                 if (mma8) {
@@ -629,272 +629,282 @@ __global__ void __launch_bounds__(kThreads, 1) attn_kernel(const AttnParams p) {
     p.trace.mark(1);
 
     // =============================== pass 2: select, gather, reduce ================================
+    // Two pieces at a time, half of the warps each: a block of the flat cut that spans two segments would otherwise go through the
+    // chain of waits, loads and reductions twice and finish last (eight sequences x 32768: the last block ten microseconds behind
+    // the median one).
     {
+        struct Piece {
+            int seg, b, g, L, lo, tb, te, off, npieces;
+            bool ident;
+        };
+        auto piece_at = [&](int64_t f, int seg) {
+            Piece c;
+            const int sb = segoff[seg], se = segoff[seg + 1];
+            c.seg = seg;
+            c.L = se - sb;
+            c.tb = static_cast<int>(f - sb);
+            c.te = static_cast<int>((f1 < se ? f1 : se) - sb);
+            c.b = seg / p.n_kv;
+            c.g = seg - c.b * p.n_kv;
+            c.lo = seq_len(c.b) - c.L;
+            c.off = static_cast<int>(f - f0) - c.tb;
+            c.ident = p.k_attn >= c.L;
+            c.npieces = pieces_of(seg);
+            return c;
+        };
         int64_t f = f0;
-        for (int seg = seg0, ord = 0; f < f1; ++seg, ++ord) {
-            const int sb = segoff[seg], se = segoff[seg + 1], L = se - sb;
-            const int tb = static_cast<int>(f - sb);
-            const int te = static_cast<int>((f1 < se ? f1 : se) - sb);
-            const int b = seg / p.n_kv, g = seg - b * p.n_kv;
-            const int lo = seq_len(b) - L;
-            const int off = static_cast<int>(f - f0) - tb;
-            const bool ident = p.k_attn >= L;
-            const int npieces = pieces_of(seg);
-            for (int i = tid; i < GQ * hd; i += kThreads) qs[i] = p.q[(static_cast<int64_t>(b) * p.n_q + g * GQ) * hd + i];
-            if (tid < GQ) sel_n[tid] = 0;
-            if (ord >= kZc && tid == 0)
-                s_z = ident ? 0.0 : (p.zs != nullptr ? p.zs[b] : -normcdfinv(static_cast<double>(p.k_attn) / static_cast<double>(L)));
-            __syncthreads();
-            if (warp < GQ) {        // theta of this head once every piece of the segment has arrived
-                double sa, sq;
+        for (int seg = seg0, ord = 0; f < f1;) {
+            const int np = f1 > segoff[seg + 1] ? 2 : 1;
+            const bool second = np == 2 && warp >= kWarps / 2;         // the warp's piece
+            const int wz = second ? 1 : 0, wl = second ? warp - kWarps / 2 : warp, nw = kWarps / np;
+            const Piece c = piece_at(second ? segoff[seg + 1] : f, seg + wz);
+            const bool more = (np == 2 ? segoff[seg + 2] : segoff[seg + 1]) < f1;
+            if (ord > 0 || more)           // more than two pieces: their queries are no longer where pass 1 put them
+                for (int i = tid; i < np * GQ * hd; i += kThreads) {
+                    const int z = i >= GQ * hd, bb = (seg + z) / p.n_kv, gg = seg + z - bb * p.n_kv;
+                    qs0[((ord + z) & 1) * GQ * hd + i - z * GQ * hd] = p.q[(static_cast<int64_t>(bb) * p.n_q + gg * GQ) * hd + i - z * GQ * hd];
+                }
+            if (tid < 2 * GQ) sel_n[tid / GQ][tid % GQ] = 0;
+            if (wl < GQ) {          // theta of this head once every piece of the segment has arrived
+                double sa, sq, z = 0.0;
                 float smax;
-                const bool ok = cells_wait_max_w<kAttnWays>(cells + static_cast<size_t>(b * p.n_q + g * GQ + warp) * kAttnWays,
-                                                            static_cast<unsigned>(npieces), sa, sq, smax, p.hdr);
+                // the quantile under the wait for the other blocks (a double-precision inverse takes a microsecond)
+                if (!c.ident) z = p.zs != nullptr ? p.zs[c.b] : -normcdfinv(static_cast<double>(p.k_attn) / static_cast<double>(c.L));
+                const bool ok = cells_wait_max_w<kAttnWays>(cells + static_cast<size_t>(c.b * p.n_q + c.g * GQ + wl) * kAttnWays,
+                                                            static_cast<unsigned>(c.npieces), sa, sq, smax, p.hdr);
                 if (lane == 0) {
                     if (!ok) s_fail = 1;
                     if (ok && p.check_finite && !(isfinite(sa) && isfinite(sq))) atomicCAS(&p.hdr->status, SPARK_OK, SPARK_ERR_NONFINITE);
                     float th = -INFINITY;
-                    if (!ident) {
-                        const double z = ord < kZc ? zcache[ord] : s_z;
-                        const double n = static_cast<double>(L), mean = sa / n;
+                    if (!c.ident) {
+                        const double n = static_cast<double>(c.L), mean = sa / n;
                         double var = (sq - sa * mean) / (n - 1.0);
                         var = var > 0.0 ? var : 0.0;
                         th = static_cast<float>(mean + sqrt(var) * z);
                     }
-                    theta_s[warp] = th;
-                    smax_s[warp] = smax;
-                    if (tb == 0 && p.theta != nullptr) p.theta[b * p.n_q + g * GQ + warp] = th;
+                    theta_s[wz][wl] = th;
+                    smax_s[wz][wl] = smax;
+                    if (c.tb == 0 && p.theta != nullptr) p.theta[c.b * p.n_q + c.g * GQ + wl] = th;
                 }
             }
             __syncthreads();
             if (s_fail) return;
             if (ord == 0) p.trace.mark(2);
-            const KT* k2base = k2c + cseg(seg) * p.cap * d2;
-            const KT* vbase = vc + cseg(seg) * p.cap * hd;
-            // In this pass warp w serves query head w % GQ; the kWarps / GQ warps of a head split the
-            // piece's tokens into contiguous runs (multiples of 32 tokens).
-            constexpr int NSUB = kWarps / GQ;
-            const int hq = warp % GQ, wsub = warp / GQ;
+            const KT* k2base = k2c + cseg(c.seg) * p.cap * d2;
+            const KT* vbase = vc + cseg(c.seg) * p.cap * hd;
+            // In this pass a warp serves query head wl % GQ; the warps of a head split the piece's tokens into contiguous runs
+            // (multiples of 32 tokens).
+            constexpr int kSub = kWarps / GQ;
+            const int hq = wl % GQ, wsub = wl / GQ, nsub = np == 2 ? kSub / 2 : kSub, sub_bits = __ffs(nsub) - 1;
+            const int tb = c.tb, te = c.te, lo = c.lo;
+            const bool ident = c.ident;
             int w0, w1;
             {
                 const int n = te - tb;
-                const int cw = (((n + NSUB - 1) / NSUB) + 31) & ~31;
+                const int cw = (((n + nsub - 1) >> sub_bits) + 31) & ~31;
                 w0 = tb + wsub * cw;
                 w1 = w0 + cw;
                 if (w0 > te) w0 = te;
                 if (w1 > te) w1 = te;
             }
-            const float th = theta_s[hq], smax = smax_s[hq];
-            const int bh = b * p.n_q + g * GQ + hq;
+            const float th = theta_s[wz][hq], smax = smax_s[wz][hq];
+            const int bh = c.b * p.n_q + c.g * GQ + hq;
+            const float* qs = qs0 + ((ord + wz) & 1) * GQ * hd;
             float q2[8];
 #pragma unroll
             for (int e = 0; e < 8; ++e) q2[e] = hl < nc2 ? qs[hq * hd + r + hl * 8 + e] : 0.f;
             float l_w = 0.f, acc[8];
 #pragma unroll
             for (int e = 0; e < 8; ++e) acc[e] = 0.f;
-            const float* srow = sc + static_cast<size_t>(hq) * ntok + off;
-            // the k2c and vc rows of up to four surviving tokens (tk: token inside the window), requested together
-            auto gather4 = [&](const int (&tk)[4], const bool (&v)[4], const float (&av)[4]) {
-                Row8<KT> kw[2], vw[4];
-                [[maybe_unused]] float ksc[2] = {1.f, 1.f}, vsc[4] = {1.f, 1.f, 1.f, 1.f};      // row scales of an FP8 cache
+            const float* srow = sc + static_cast<size_t>(hq) * ntok + c.off;
+            // The k2c and vc rows of nv <= kGather surviving tokens (tk: token inside the window), requested together.  Half h of the
+            // warp reads the k2c rows of entries 2 i + h, and lane 16 h + i makes that entry's weight (its token and s - s_max in
+            // tok_l and a_l): an exponential and a softplus per trip instead of one per entry.
+            constexpr int kGather = sizeof(KT) == 4 ? 4 : 8;
+            const int entry = 2 * (lane & (kGather / 2 - 1)) + half;         // the entry whose weight this lane makes
+            const bool holder = hl < kGather / 2;
+            auto gather = [&](const int (&tk)[kGather], int nv, int tok_l, float a_l) {
+                Row8<KT> kw[kGather / 2], vw[kGather];
 #pragma unroll
-                for (int i = 0; i < 2; ++i) {      // half h reads the k2c rows of entries h and h + 2
-                    const bool vv = half ? v[1 + 2 * i] : v[2 * i];
-                    const int tt = half ? tk[1 + 2 * i] : tk[2 * i];
-                    if (vv && hl < nc2) kw[i].load(k2base + static_cast<int64_t>(lo + tt) * d2, hl);
+                for (int i = 0; i < kGather / 2; ++i) {
+                    if (2 * i + half < nv && hl < nc2) kw[i].load(k2base + static_cast<int64_t>(lo + (half ? tk[2 * i + 1] : tk[2 * i])) * d2, hl);
                     else kw[i].zero();
-                    if constexpr (sizeof(KT) == 1) ksc[i] = vv ? __ldg(p.k2s + cseg(seg) * p.cap + lo + tt) : 1.f;
                 }
 #pragma unroll
-                for (int i = 0; i < 4; ++i) {
-                    if (v[i] && lane < ncv) vw[i].load(vbase + static_cast<int64_t>(lo + tk[i]) * hd, lane);
+                for (int i = 0; i < kGather; ++i) {
+                    if (i < nv && lane < ncv) vw[i].load(vbase + static_cast<int64_t>(lo + tk[i]) * hd, lane);
                     else vw[i].zero();
-                    if constexpr (sizeof(KT) == 1) vsc[i] = v[i] ? __ldg(p.vs + cseg(seg) * p.cap + lo + tk[i]) : 1.f;
                 }
-                float gt[4];
+                [[maybe_unused]] float ksc = 1.f, vsc = 1.f;                 // row scales of an FP8 cache
+                if constexpr (sizeof(KT) == 1)
+                    if (holder && entry < nv) {
+                        ksc = __ldg(p.k2s + cseg(c.seg) * p.cap + lo + tok_l);
+                        vsc = __ldg(p.vs + cseg(c.seg) * p.cap + lo + tok_l);
+                    }
+                float x = 0.f;
 #pragma unroll
-                for (int i = 0; i < 2; ++i) {
+                for (int i = 0; i < kGather / 2; ++i) {
+                    if (2 * i >= nv) break;
                     float wf[8];
                     kw[i].unpack(wf);
-                    const float gate = softplus(sizeof(KT) == 1 ? ksc[i] * half_sum(dot8r(wf, q2)) : half_sum(dot8r(wf, q2)));
-                    gt[2 * i] = __shfl_sync(kFull, gate, 0);
-                    gt[2 * i + 1] = __shfl_sync(kFull, gate, 16);
+                    const float sum = half_sum(dot8r(wf, q2));
+                    if (entry >> 1 == i) x = sum;
                 }
-                float wt[4];
+                const float pe = holder && entry < nv && a_l != -INFINITY ? expf(a_l) : 0.f;
+                l_w += pe;
+                const float wgt = pe * softplus(ksc * x) * vsc;              // unselected rows of the dense comparator get weight 0 * gate
 #pragma unroll
-                for (int i = 0; i < 4; ++i) {
-                    const float pe = av[i] == -INFINITY ? 0.f : expf(av[i]);
-                    l_w += pe;
-                    wt[i] = pe * gt[i];         // unselected rows of the dense comparator get weight 0 * gate
-                    if constexpr (sizeof(KT) == 1) wt[i] *= vsc[i];
-                }
-#pragma unroll
-                for (int i = 0; i < 4; ++i) {
+                for (int i = 0; i < kGather; ++i) {
+                    if (i >= nv) break;
+                    const float wt = __shfl_sync(kFull, wgt, (i & 1) * 16 + (i >> 1));
                     float fv[8];
                     vw[i].unpack(fv);
 #pragma unroll
-                    for (int e = 0; e < 8; ++e) acc[e] = fmaf(wt[i], fv[e], acc[e]);
+                    for (int e = 0; e < 8; ++e) acc[e] = fmaf(wt, fv[e], acc[e]);
                 }
             };
-            int* ltok = sel_tok + static_cast<size_t>(hq) * ntok;
-            float* la = sel_a + static_cast<size_t>(hq) * ntok;
-            bool listed = false;
-            if constexpr (M16 || sizeof(K1T) == 1) {
-            if (p.sel_list && (M16 || p.long_share)) {
-                listed = true;
-                // Two sweeps over the warp's scores, four 32-token steps per trip with their loads issued together (a step per
-                // trip left every warp waiting on its own chain of load, compare and vote: 0.3 us per step).  The first sweep
-                // counts what the warp will list; a single shared-memory atomic reserves that many entries of the head's list.
-                int mine = 0;
-#pragma unroll 1
-                for (int base = w0; base < w1; base += 128) {
-                    float sv[4];
+            // a piece's part of a head's list has the places of its scores
+            int* ltok = sel_tok + static_cast<size_t>(hq) * ntok + c.off + tb;
+            float* la = sel_a + static_cast<size_t>(hq) * ntok + c.off + tb;
+            // Adds a warp's survivors to the head's count; returns where this lane's first one goes in the caller's list.
+            auto count_base = [&](int before, int total) -> int64_t {
+                int base = 0;
+                if (lane == 0 && total > 0) base = atomicAdd(&p.count[bh], total);
+                return static_cast<int64_t>(__shfl_sync(kFull, base, 0)) + before;
+            };
+            auto put_idx = [&](int64_t pos, int t) {
+                if (pos < p.idx_cap) p.idx[static_cast<int64_t>(bh) * p.idx_cap + pos] = lo + t;
+                else atomicCAS(&p.hdr->status, SPARK_OK, SPARK_ERR_OVERFLOW);
+            };
+            auto scan = [&](int v, int& total) -> int {         // sum over the lanes before this one
+                int incl = v;
 #pragma unroll
-                    for (int u = 0; u < 4; ++u) {
-                        const int t = base + 32 * u + lane;
-                        sv[u] = t < w1 ? srow[t] : -INFINITY;
-                    }
-#pragma unroll
-                    for (int u = 0; u < 4; ++u) {
-                        const bool valid = base + 32 * u + lane < w1;
-                        mine += __popc(__ballot_sync(kFull, valid && (p.dense || ident || sv[u] > th)));
-                    }
+                for (int o = 1; o < 32; o <<= 1) {
+                    const int x = __shfl_up_sync(kFull, incl, o);
+                    if (lane >= o) incl += x;
                 }
-                int lpos = 0;
-                if (lane == 0 && mine > 0) lpos = atomicAdd(&sel_n[hq], mine);
-                lpos = __shfl_sync(kFull, lpos, 0);
+                total = __shfl_sync(kFull, incl, 31);
+                return incl - v;
+            };
+            if (p.sel_list) {
+                // The survivors of the whole piece go to one list per head, from which the head's warps then take equal shares: a warp
+                // that found many does not make the block wait for a second round of loads while others found none.  A lane keeps its
+                // survivors among up to 1024 tokens of the warp as bits and the lanes' counts are scanned once (with a vote per 32 tokens,
+                // twice over the scores: 4.7 us at 690 tokens a warp).
 #pragma unroll 1
-                for (int base = w0; base < w1; base += 128) {
-                    float sv[4];
+                for (int base = w0; base < w1; base += 1024) {
+                    unsigned mask, all;
+                    int total, before;
+                    if (w1 - base <= 32) {                                         // a token per lane
+                        const bool valid = base + lane < w1;
+                        mask = valid && (ident || srow[base + lane] > th) ? 1u : 0u;
+                        all = p.dense ? (valid ? 1u : 0u) : mask;
+                        const unsigned votes = __ballot_sync(kFull, all != 0u);
+                        total = __popc(votes);
+                        before = __popc(votes & ((1u << lane) - 1u));
+                    } else {
+                        mask = 0u;
+#pragma unroll 1
+                        for (int u0 = 0; u0 < 32 && base + 32 * u0 < w1; u0 += 8) {
+                            float sv[8];
 #pragma unroll
-                    for (int u = 0; u < 4; ++u) {
-                        const int t = base + 32 * u + lane;
-                        sv[u] = t < w1 ? srow[t] : 0.f;
-                    }
+                            for (int u = 0; u < 8; ++u) {
+                                const int t = base + 32 * (u0 + u) + lane;
+                                sv[u] = t < w1 ? srow[t] : 0.f;
+                            }
 #pragma unroll
-                    for (int u = 0; u < 4; ++u) {
-                        const int t = base + 32 * u + lane;
-                        const bool valid = t < w1;
-                        const float s = sv[u];
-                        const bool sel = valid && (ident || s > th);
-                        const float a = sel ? s - smax : -INFINITY;        // softmax is shift-invariant: the head's largest score is the reference
-                        const unsigned bsel = __ballot_sync(kFull, sel);
-                        const unsigned bal = p.dense ? __ballot_sync(kFull, valid) : bsel;
-                        if (p.count != nullptr && bsel != 0u) {
-                            int cbase = 0;
-                            if (lane == 0) cbase = atomicAdd(&p.count[bh], __popc(bsel));
-                            cbase = __shfl_sync(kFull, cbase, 0);
-                            if (sel && p.idx != nullptr) {
-                                const int64_t pos = static_cast<int64_t>(cbase) + __popc(bsel & ((1u << lane) - 1u));
-                                if (pos < p.idx_cap) p.idx[static_cast<int64_t>(bh) * p.idx_cap + pos] = lo + t;
-                                else atomicCAS(&p.hdr->status, SPARK_OK, SPARK_ERR_OVERFLOW);
+                            for (int u = 0; u < 8; ++u) {
+                                const bool valid = base + 32 * (u0 + u) + lane < w1;
+                                mask |= valid && (ident || sv[u] > th) ? 1u << (u0 + u) : 0u;
                             }
                         }
-                        // The survivors of the whole piece go to one list per head, from which the head's warps then take four
-                        // entries each: a warp that found many does not make the block wait for a second round of loads while
-                        // others found none.
-                        if ((bal >> lane) & 1u) {
-                            const int pos = lpos + __popc(bal & ((1u << lane) - 1u));
-                            ltok[pos] = t;
-                            la[pos] = a;
-                        }
-                        lpos += __popc(bal);
+                        const int left = (w1 - base - lane + 31) >> 5;             // this lane's tokens of the window
+                        all = p.dense ? (left >= 32 ? 0xffffffffu : (1u << (left > 0 ? left : 0)) - 1u) : mask;
+                        before = scan(__popc(all), total);
+                    }
+                    int at = 0;
+                    if (lane == 0 && total > 0) at = atomicAdd(&sel_n[wz][hq], total);
+                    at = __shfl_sync(kFull, at, 0) + before;
+                    for (unsigned m = all; m != 0u; m &= m - 1u, ++at) {
+                        const int u = __ffs(m) - 1, t = base + 32 * u + lane;
+                        ltok[at] = t;
+                        la[at] = mask >> u & 1u ? srow[t] - smax : -INFINITY;      // softmax is shift-invariant: the head's largest score is the reference
+                    }
+                    if (p.count != nullptr) {
+                        int sel_total = total, sel_before = before;
+                        if (p.dense) sel_before = scan(__popc(mask), sel_total);
+                        int64_t pos = count_base(sel_before, sel_total);
+                        if (p.idx != nullptr)
+                            for (unsigned m = mask; m != 0u; m &= m - 1u, ++pos) put_idx(pos, base + 32 * (__ffs(m) - 1) + lane);
                     }
                 }
-            }
-            }
-            if (!listed) {
+            } else {
 #pragma unroll 1
             for (int base = w0; base < w1; base += 32) {
                 const int t = base + lane;
                 const bool valid = t < w1;
                 const float s = valid ? srow[t] : 0.f;
                 const bool sel = valid && (ident || s > th);
-                const float a = sel ? s - smax : -INFINITY;        // softmax is shift-invariant: the head's largest score is the reference
+                const float a = sel ? s - smax : -INFINITY;
                 const unsigned bsel = __ballot_sync(kFull, sel);
                 unsigned bal = p.dense ? __ballot_sync(kFull, valid) : bsel;
                 if (p.count != nullptr && bsel != 0u) {
-                    int cbase = 0;
-                    if (lane == 0) cbase = atomicAdd(&p.count[bh], __popc(bsel));
-                    cbase = __shfl_sync(kFull, cbase, 0);
-                    if (sel && p.idx != nullptr) {
-                        const int64_t pos = static_cast<int64_t>(cbase) + __popc(bsel & ((1u << lane) - 1u));
-                        if (pos < p.idx_cap) p.idx[static_cast<int64_t>(bh) * p.idx_cap + pos] = lo + t;
-                        else atomicCAS(&p.hdr->status, SPARK_OK, SPARK_ERR_OVERFLOW);
-                    }
+                    const int64_t pos = count_base(__popc(bsel & ((1u << lane) - 1u)), __popc(bsel));
+                    if (sel && p.idx != nullptr) put_idx(pos, t);
                 }
-                if (p.sel_list) {
-                    // The survivors of the whole piece go to one list per head, from which the head's warps
-                    // then take four entries each: a warp that found many does not make the block wait for a
-                    // second round of loads while others found none.
-                    if (bal != 0u) {
-                        int pos0 = 0;
-                        if (lane == 0) pos0 = atomicAdd(&sel_n[hq], __popc(bal));
-                        pos0 = __shfl_sync(kFull, pos0, 0);
-                        if ((bal >> lane) & 1u) {
-                            const int pos = pos0 + __popc(bal & ((1u << lane) - 1u));
-                            ltok[pos] = t;
-                            la[pos] = a;
-                        }
-                    }
-                    continue;
-                }
-                while (bal != 0u) {          // four listed tokens per trip: their rows are requested together
-                    int tk[4];
-                    bool v[4];
-                    float av[4];
+                while (bal != 0u) {          // kGather listed tokens per trip
+                    int tk[kGather], nv = 0, src = 0;
 #pragma unroll
-                    for (int i = 0; i < 4; ++i) {
-                        v[i] = bal != 0u;
-                        const int l = v[i] ? __ffs(bal) - 1 : 0;
-                        if (v[i]) bal &= bal - 1u;
-                        const float x = __shfl_sync(kFull, a, l);
-                        av[i] = v[i] ? x : -INFINITY;
+                    for (int i = 0; i < kGather; ++i) {
+                        const int l = bal != 0u ? __ffs(bal) - 1 : 0;
+                        nv += bal != 0u ? 1 : 0;
+                        bal &= bal - 1u;
+                        if (entry == i) src = l;
                         tk[i] = base + l;
                     }
-                    gather4(tk, v, av);
+                    gather(tk, nv, base + src, __shfl_sync(kFull, a, src));
                 }
             }
             }
             if (p.sel_list) {
                 __syncthreads();
-                const int n = sel_n[hq];
+                const int n = sel_n[wz][hq], e1 = n * (wsub + 1) >> sub_bits;
 #pragma unroll 1
-                for (int e0 = wsub * 4; e0 < n; e0 += NSUB * 4) {
-                    int tk[4];
-                    bool v[4];
-                    float av[4];
+                for (int e0 = n * wsub >> sub_bits; e0 < e1; e0 += kGather) {
+                    int tk[kGather];
+                    const int nv = min(e1 - e0, kGather);
 #pragma unroll
-                    for (int i = 0; i < 4; ++i) {
-                        v[i] = e0 + i < n;
-                        tk[i] = v[i] ? ltok[e0 + i] : 0;
-                        av[i] = v[i] ? la[e0 + i] : -INFINITY;
-                    }
-                    gather4(tk, v, av);
+                    for (int i = 0; i < kGather; ++i) tk[i] = i < nv ? ltok[e0 + i] : 0;
+                    const bool in = entry < nv;
+                    gather(tk, nv, in ? ltok[e0 + entry] : 0, in ? la[e0 + entry] : -INFINITY);
                 }
             }
-            // ---- add the block's sum of weights and weighted values to the heads' accumulators ----------
+            // ---- add the block's sums of weights and weighted values to the heads' accumulators ----------
             {
                 float* wp = wpart + warp * pstride;
+                l_w += __shfl_xor_sync(kFull, l_w, 16);          // the holders' sums
+#pragma unroll
+                for (int o = kGather / 4; o > 0; o >>= 1) l_w += __shfl_xor_sync(kFull, l_w, o);
                 if (lane == 0) wp[1] = l_w;
                 if (lane < ncv) {
 #pragma unroll
                     for (int e = 0; e < 8; ++e) wp[kPartPad + lane * 8 + e] = acc[e];
                 }
                 __syncthreads();
-                for (int i = tid; i < GQ * (hd / 4); i += kThreads) {
-                    const int h = i / (hd / 4), d4 = i - h * (hd / 4);
+                for (int i = tid; i < np * GQ * (hd / 4); i += kThreads) {
+                    const int zh = i / (hd / 4), z = zh / GQ, h = zh - z * GQ, d4 = i - zh * (hd / 4);
                     float4 sum = make_float4(0.f, 0.f, 0.f, 0.f);
                     float l = 0.f;
 #pragma unroll
-                    for (int u = 0; u < NSUB; ++u) {
-                        const float* e = wpart + (u * GQ + h) * pstride;
+                    for (int u = 0; u < kSub; ++u) {
+                        if (u >= nsub) break;
+                        const float* e = wpart + (z * nw + u * GQ + h) * pstride;
                         const float4 x = *reinterpret_cast<const float4*>(e + kPartPad + d4 * 4);
                         sum.x += x.x; sum.y += x.y; sum.z += x.z; sum.w += x.w;
                         l += e[1];
                     }
                     if (l > 0.f || p.dense) {
-                        const int64_t hb = static_cast<int64_t>(b) * p.n_q + g * GQ + h;
+                        const int64_t hb = static_cast<int64_t>(seg + z) * GQ + h;             // = sequence n_q + KV head GQ + h
                         red_add_v4(p.o + hb * hd + d4 * 4, sum.x, sum.y, sum.z, sum.w);
                         if (d4 == 0) atomicAdd(&p.lsum[hb], l);
                     }
@@ -903,35 +913,35 @@ __global__ void __launch_bounds__(kThreads, 1) attn_kernel(const AttnParams p) {
             }
             // ---- the block that completes a segment last divides by the sum of weights -----------------
             if (!p.defer) {
-                if (tid == 0) {
+                if (lane == 0 && wl == 0) {
                     __threadfence();
-                    const unsigned prev = atom_add_acqrel_u32(&p.hdr->seg_done[seg], 1u);
-                    const int last = prev == static_cast<unsigned>(npieces - 1);
-                    if (last) p.hdr->seg_done[seg] = 0u;
-                    s_last = last;
+                    const unsigned prev = atom_add_acqrel_u32(&p.hdr->seg_done[c.seg], 1u);
+                    const int last = prev == static_cast<unsigned>(c.npieces - 1);
+                    if (last) p.hdr->seg_done[c.seg] = 0u;
+                    s_last[wz] = last;
                 }
                 __syncthreads();
-                if (s_last) {
+                for (int z = 0; z < np; ++z) {
+                    if (!s_last[z]) continue;
                     for (int i = tid; i < GQ * hd; i += kThreads) {
                         const int h = i / hd;
-                        const int64_t hb = static_cast<int64_t>(b) * p.n_q + g * GQ + h;
+                        const int64_t hb = static_cast<int64_t>(seg + z) * GQ + h;
                         const float l = __ldcg(&p.lsum[hb]);
                         float* od = p.o + hb * hd + (i - h * hd);
                         const float v = __ldcg(od);
                         *od = l > 0.f ? v / l : 0.f;
                     }
+                    // every piece of the segment has read the cells by now: leave them zero for the next launch
+                    if (tid < GQ * kAttnWays) {
+                        SumCell* cell = cells + static_cast<size_t>(seg + z) * GQ * kAttnWays + tid;
+                        cell->s1 = 0.0; cell->s2 = 0.0; cell->count = 0u; cell->pad[0] = 0u;
+                    }
                 }
-            } else if (tid == 0) {
-                s_last = 0;
             }
             __syncthreads();
-            // every piece of the segment has read the cells by now: leave them zero for the next launch
-            if (s_last && tid < GQ * kAttnWays) {
-                SumCell* c = cells + static_cast<size_t>(b * p.n_q + g * GQ) * kAttnWays + tid;
-                c->s1 = 0.0; c->s2 = 0.0; c->count = 0u; c->pad[0] = 0u;
-            }
-            __syncthreads();
-            f = sb + te;
+            f = np == 2 && !more ? f1 : segoff[seg + np];
+            seg += np;
+            ord += np;
         }
     }
     p.trace.mark(3);
@@ -1020,7 +1030,7 @@ int attn_launch(spark_ctx* ctx, const float* q, const void* k1c, const void* k2c
     if (static_cast<size_t>(B * n_q) * kAttnWays * sizeof(SumCell) > cells_b) return SPARK_ERR_UNSUPPORTED;
     const size_t part_b = round_up(static_cast<size_t>(B * n_q) * 4, 256);     // sums of weights (standalone calls)
     const size_t ns_pad = (static_cast<size_t>(B * n_kv) + 1 + 3) & ~static_cast<size_t>(3);
-    const size_t smem_fixed = ns_pad * 4 + static_cast<size_t>(gq * hd) * 4 + static_cast<size_t>(kWarps) * (hd + kPartPad) * 4;
+    const size_t smem_fixed = ns_pad * 4 + static_cast<size_t>(2 * gq * hd) * 4 + static_cast<size_t>(kWarps) * (hd + kPartPad) * 4;
     const size_t smem_limit = static_cast<size_t>(ctx->max_smem_optin - 8192);
     if (smem_fixed > smem_limit) return SPARK_ERR_UNSUPPORTED;
     // room for the segment-aligned cut, whose shares are uneven, when everything still fits shared memory
@@ -1062,8 +1072,7 @@ int attn_launch(spark_ctx* ctx, const float* q, const void* k1c, const void* k2c
     // measured: the tensor-core pass wins from about 450 tokens a block on (16384 tokens, one sequence: 16.3 -> 15.5 us; eight
     // sequences x 32768: 77.2 -> 71.9) but gives up the rows requested before the kernel ahead has finished, which a layer
     // call of one 9B-shaped sequence (443 tokens a block) still wants: from 800 tokens a block
-    p.long_share = ntok >= 800 ? 1 : 0;
-    p.mma_pass = (kvdtype == SPARK_BF16 && k1s == nullptr && p.long_share) ? 1 : 0;
+    p.mma_pass = (kvdtype == SPARK_BF16 && k1s == nullptr && ntok >= 800) ? 1 : 0;
     p.scores = reinterpret_cast<float*>(ctx->scratch + cells_b + part_b);
     p.ntok = static_cast<int>(ntok);
     p.sc_smem = sc_smem ? 1 : 0;
