@@ -1,13 +1,14 @@
-// Dense projection for 5..64 tokens with bf16 weights on the fifth-generation tensor cores:
+// Dense projection for 2..64 tokens with bf16 weights on the fifth-generation tensor cores:
 // y[b][:] = Wt . f(x[b][:]) (+ y_add[b][:]), f = optional division per group, optional RMSNorm -- the
 // decoder layer's QKV and output projections for a batch or a chunk of a prompt, the LM head of a batch.  Two kernels:
-//   prep   f(x) -> two bf16 terms (x = hi + lo, 16 significant bits) in the workspace; the addend (or 0) into those output
-//          tiles that two or more blocks of the GEMM share; the caller's clear-region side job
+//   prep   f(x) -> two bf16 terms (x = hi + lo, 16 significant bits) in the workspace, three (all 24 bits) for up to four tokens;
+//          the addend (or 0) into those output tiles that two or more blocks of the GEMM share; the caller's clear-region side job
 //   gemm   the weight-streaming GEMM of stream_gemm.cuh, any number of output rows and any n_in (multiple of 8; TMA fills what
 //          lies outside with zeros); a tile that one block holds whole is stored, a shared one reduced into y
 // Row counts that are no multiple of 128 used to take the mma.sync kernels: 105401 x 2048, 64 tokens, 375 -> 81 us; 5 tokens
 // 76 -> 70.  The 256000 x 2304 head went from whole tiles per block and a wave of blocks per 148 of them to a persistent
-// sequence: 64 tokens 256 -> 201 us, 8 tokens 201 -> 181.
+// sequence: 64 tokens 256 -> 201 us, 8 tokens 201 -> 181.  Two to four tokens were bound by the plain ALUs: 256000 x 2304, 2 tokens,
+// 261 -> 177 us; 16000 x 2304 26.3 -> 18.2; 4096 x 2304 12.4 -> 9.7; 1000 x 1000 6.2 both.
 #include "kernels.h"
 #include "stream_gemm.cuh"
 
@@ -30,12 +31,13 @@ struct GemmParams {
     int x_div_group;
     uint4* zero_ptr;
     int zero_n16;
-    __nv_bfloat16* xs;       // [2 * ntok][n_in]
+    __nv_bfloat16* xs;       // [xrows][n_in]
     StreamPlan sp;
     WsHeader* hdr;
 };
 
 // Four blocks per (padded) token row, a quarter of the row each.
+template <bool FEW>
 __global__ void __launch_bounds__(256) gemm_tc_prep_kernel(const GemmParams p) {
     __shared__ float red[8];
     const int n = blockIdx.x / kGemmPrepSplit, qr = blockIdx.x % kGemmPrepSplit, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
@@ -98,24 +100,33 @@ __global__ void __launch_bounds__(256) gemm_tc_prep_kernel(const GemmParams p) {
             const float4 w = reinterpret_cast<const float4*>(p.norm_w)[i];
             v = make_float4(v.x * sc * w.x, v.y * sc * w.y, v.z * sc * w.z, v.w * sc * w.w);
         }
-        unsigned h01, h23, l01, l23;
-        split_pair(v.x, v.y, h01, l01);
-        split_pair(v.z, v.w, h23, l23);
-        reinterpret_cast<uint2*>(p.xs + static_cast<int64_t>(n) * n_in)[i] = make_uint2(h01, h23);
-        reinterpret_cast<uint2*>(p.xs + static_cast<int64_t>(p.sp.ntok + n) * n_in)[i] = make_uint2(l01, l23);
+        uint2 h, m, l;
+        uint2* row = reinterpret_cast<uint2*>(p.xs + static_cast<int64_t>(n) * n_in) + i;
+        const int64_t term = static_cast<int64_t>(p.sp.ntok) * (n_in / 4);
+        if (FEW) {
+            split_pair3(v.x, v.y, h.x, m.x, l.x);
+            split_pair3(v.z, v.w, h.y, m.y, l.y);
+            row[2 * term] = l;
+        } else {
+            split_pair(v.x, v.y, h.x, m.x);
+            split_pair(v.z, v.w, h.y, m.y);
+        }
+        row[0] = h;
+        row[term] = m;
     }
 }
 
+template <bool FEW>
 __global__ void __launch_bounds__(kTcThreads, 1)
 gemm_tc_kernel(const GemmParams p, const __grid_constant__ CUtensorMap map_w, const __grid_constant__ CUtensorMap map_x) {
     extern __shared__ unsigned char tc_raw[];
     __shared__ StreamShared sh;
-    stream_gemm<0>(p.sp, sh, tc_raw, &map_w, &map_x, p.hdr, [] {}, [&](int tile, bool whole, int r, int n0, const float (&v)[16]) {
+    stream_gemm<FEW ? kStreamFew : 0>(p.sp, sh, tc_raw, &map_w, &map_x, p.hdr, [] {}, [&](int tile, bool whole, int r, int n0, const float (&v)[16]) {
         const int row = tile * kStreamRows + r;
         if (row >= p.n_out) return;
         const int64_t at = static_cast<int64_t>(n0) * p.n_out + row;
 #pragma unroll
-        for (int i = 0; i < 16; ++i)
+        for (int i = 0; i < (FEW ? 4 : 16); ++i)
             if (n0 + i < p.B) {
                 float* y = p.y + at + static_cast<int64_t>(i) * p.n_out;
                 if (!whole) atomicAdd(y, v[i]);
@@ -130,15 +141,16 @@ namespace spark {
 
 // SPARK_ERR_WORKSPACE = shape or workspace not served by this path (the caller falls back).
 int gemm_tc_launch(spark_ctx* ctx, const GemvArgs& a, cudaStream_t stream) {
-    if (a.wdtype != SPARK_BF16 || a.B < 5 || a.B > kGemmMaxTok || (a.n_in & 7) != 0 || a.n_in < kChunk) return SPARK_ERR_WORKSPACE;
+    if (a.wdtype != SPARK_BF16 || a.B < 2 || a.B > kGemmMaxTok || (a.n_in & 7) != 0 || a.n_in < kChunk) return SPARK_ERR_WORKSPACE;
     if ((reinterpret_cast<uintptr_t>(a.Wt) & 15u) != 0) return SPARK_ERR_WORKSPACE;
     GemmParams p;
+    const bool few = a.B <= 4;
     const int64_t call = (a.n_in + kChunk - 1) / kChunk, tiles = (a.n_out + kStreamRows - 1) / kStreamRows;
     if (tiles * call >= (1LL << 30)) return SPARK_ERR_WORKSPACE;
     const size_t limit = static_cast<size_t>(ctx->max_smem_optin) - sizeof(StreamShared) - 64;
-    if (!stream_plan(p.sp, ctx->num_sms, static_cast<int>(tiles), static_cast<int>(call), static_cast<int>(a.B), limit)) return SPARK_ERR_WORKSPACE;
+    if (!stream_plan(p.sp, ctx->num_sms, static_cast<int>(tiles), static_cast<int>(call), static_cast<int>(a.B), limit, false, kStreamRows, few)) return SPARK_ERR_WORKSPACE;
     // the split input sits behind the attention's cells, where the FFN chunk path keeps its own (neither outlives its call)
-    const size_t xb = static_cast<size_t>(2) * p.sp.ntok * a.n_in * 2;
+    const size_t xb = static_cast<size_t>(p.sp.xrows) * a.n_in * 2;
     if (ctx->scratch == nullptr || ctx->scratch_bytes < kAttnCellBytes + xb) return SPARK_ERR_WORKSPACE;
 
     p.x = a.x; p.norm_w = a.norm_w; p.eps = a.rms_eps;
@@ -151,13 +163,14 @@ int gemm_tc_launch(spark_ctx* ctx, const GemvArgs& a, cudaStream_t stream) {
 
     CUtensorMap m_w, m_x;
     if (!make_map(&m_w, a.Wt, a.n_out, a.n_in, a.n_in, kStreamRows, true) ||
-        !make_map(&m_x, p.xs, 2 * p.sp.ntok, a.n_in, a.n_in, 2 * p.sp.ntok, false))
+        !make_map(&m_x, p.xs, p.sp.xrows, a.n_in, a.n_in, p.sp.xrows, false))
         return SPARK_ERR_WORKSPACE;
-    const void* kern = reinterpret_cast<const void*>(gemm_tc_kernel);
+    const void* kern = few ? reinterpret_cast<const void*>(gemm_tc_kernel<true>) : reinterpret_cast<const void*>(gemm_tc_kernel<false>);
+    const void* prep = few ? reinterpret_cast<const void*>(gemm_tc_prep_kernel<true>) : reinterpret_cast<const void*>(gemm_tc_prep_kernel<false>);
     if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(limit)) != cudaSuccess) return SPARK_ERR_CUDA;
     {
         void* args[] = {&p};
-        if (launch_kernel(ctx, reinterpret_cast<const void*>(gemm_tc_prep_kernel), static_cast<unsigned>(p.sp.ntok * kGemmPrepSplit), 256, 0, stream, false, args) != cudaSuccess)
+        if (launch_kernel(ctx, prep, static_cast<unsigned>((few ? 16 : p.sp.ntok) * kGemmPrepSplit), 256, 0, stream, false, args) != cudaSuccess)
             return SPARK_ERR_CUDA;
     }
     {

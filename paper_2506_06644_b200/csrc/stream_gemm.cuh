@@ -35,7 +35,8 @@ struct StreamPlan {
     uint32_t inv_split;      // 65536 / split + 1: block / split for fewer than 65536 / split blocks
     int call;                // K chunks of a tile
     int rows;                // rows of a tile: 128, or a smaller multiple of 8 (the MMAs' other rows read whatever lies behind and are dropped)
-    int ntok;                // tokens rounded up to a multiple of 16: half of the MMAs' N; X has rows term * ntok + token
+    int ntok;                // token t's term i is row i * ntok + t of X: two terms, ntok a multiple of 16; kStreamFew: three terms, ntok = 4
+    int xrows;               // rows of X: the MMAs' N
     int stages;
     int stage_bytes;
     uint32_t tmem_cols;
@@ -61,7 +62,7 @@ inline size_t stream_slack(const StreamPlan& sp) { return 1024 + static_cast<siz
 
 // Host: fills in the plan for at most `smem_limit` bytes of dynamic shared memory.  whole: a block takes one whole tile, however many
 // there are (the caller needs whole products).  False: does not fit.
-inline bool stream_plan(StreamPlan& sp, int sms, int tiles, int call, int tokens, size_t smem_limit, bool whole = false, int rows = kStreamRows) {
+inline bool stream_plan(StreamPlan& sp, int sms, int tiles, int call, int tokens, size_t smem_limit, bool whole = false, int rows = kStreamRows, bool few = false) {
     sp.call = call;
     sp.total = tiles * call;
     sp.rows = rows;
@@ -86,8 +87,9 @@ inline bool stream_plan(StreamPlan& sp, int sms, int tiles, int call, int tokens
     sp.part = of / by;
     sp.rem = of % by;
     sp.inv_split = sp.split > 0 ? 65536u / static_cast<uint32_t>(sp.split) + 1u : 0u;
-    sp.ntok = (tokens + 15) & ~15;
-    sp.stage_bytes = (rows + 2 * sp.ntok) * kChunk * 2;
+    sp.ntok = few ? 4 : (tokens + 15) & ~15;
+    sp.xrows = few ? 16 : 2 * sp.ntok;
+    sp.stage_bytes = (rows + sp.xrows) * kChunk * 2;
     const int fit = static_cast<int>((smem_limit - stream_slack(sp)) / sp.stage_bytes);
     // more than eight stages (128 KB of weights in flight per SM, three times what the latency of HBM needs) only delays the
     // small loads of the kernel ahead that queue behind them
@@ -97,7 +99,7 @@ inline bool stream_plan(StreamPlan& sp, int sms, int tiles, int call, int tokens
     const int most = sp.per > 0 ? sp.per : sp.part + (sp.rem > 0 ? 1 : 0);
     if (sp.stages > most) sp.stages = most > 2 ? most : 2;
     uint32_t cols = 32;
-    while (cols < static_cast<uint32_t>((sp.split > 0 || sp.per == call ? 2 : 4) * sp.ntok)) cols *= 2;
+    while (cols < static_cast<uint32_t>((sp.split > 0 || sp.per == call ? 1 : 2) * sp.xrows)) cols *= 2;
     sp.tmem_cols = cols;
     return sp.stages >= 2 && cols <= 512 && tiles > 0 && call > 0;
 }
@@ -109,7 +111,8 @@ inline size_t stream_smem(const StreamPlan& sp) { return static_cast<size_t>(sp.
 //   kStreamLate     the kernel behind may start once this one has seen the end of the kernel ahead (implied by kStreamEarlyX);
 //                   otherwise at once: it only requests its weights before it waits for this kernel
 //   kStreamMN       A is stored [K][rows] (two boxes of 64 rows per K chunk)
-constexpr int kStreamEarlyX = 1, kStreamLate = 2, kStreamMN = 4;
+//   kStreamFew      up to four tokens in three bf16 terms each (x = hi + mid + lo, all 24 bits of an fp32 value): 12 of 16 rows of X
+constexpr int kStreamEarlyX = 1, kStreamLate = 2, kStreamMN = 4, kStreamFew = 8;
 
 // One block's work.  before() runs in the four epilogue warps once the kernel ahead is complete.  epi(tile, whole, row, n0, v):
 // sixteen tokens' values of one row of a tile (a whole warp calls it; rows from sp.rows on are to be dropped); `whole`: the block
@@ -117,7 +120,7 @@ constexpr int kStreamEarlyX = 1, kStreamLate = 2, kStreamMN = 4;
 template <int V, class Before, class Epi>
 __device__ __forceinline__ void stream_gemm(const StreamPlan& sp, StreamShared& sh, unsigned char* raw, const CUtensorMap* map_w,
                                             const CUtensorMap* map_x, WsHeader* hdr, Before before, Epi epi) {
-    constexpr bool kEarlyX = (V & kStreamEarlyX) != 0, kLate = (V & (kStreamEarlyX | kStreamLate)) != 0, kMN = (V & kStreamMN) != 0;
+    constexpr bool kEarlyX = (V & kStreamEarlyX) != 0, kLate = (V & (kStreamEarlyX | kStreamLate)) != 0, kMN = (V & kStreamMN) != 0, kFew = (V & kStreamFew) != 0;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const StreamPart part = stream_part(sp, blockIdx.x);
     const int n = part.n;
@@ -194,14 +197,14 @@ __device__ __forceinline__ void stream_gemm(const StreamPlan& sp, StreamShared& 
         }
     } else if (warp == 1) {
         // the whole warp walks the loop; one elected lane issues
-        const uint32_t elected = elect_lane(), idesc = instr_desc(128, 2 * sp.ntok, kMN);
+        const uint32_t elected = elect_lane(), idesc = instr_desc(128, sp.xrows, kMN);
         int s = 0, seg = 0;
         uint32_t parity = 0u;
         bool ok = true;
         for (int done = 0, len = min(n, sp.call - part.c); done < n && ok; done += len, len = min(n - done, sp.call)) {
             const int b = seg & 1;
             if (seg >= 2) ok = __all_sync(kFull, mbar_wait(smem_addr(&sh.acc_empty[b]), ((seg >> 1) & 1) ^ 1, abort_flag));
-            const uint32_t acc = tmem + static_cast<uint32_t>(b * 2 * sp.ntok);
+            const uint32_t acc = tmem + static_cast<uint32_t>(b * sp.xrows);
             tc_fence_after();
             uint32_t more = 0u;
             for (int i = 0; i < len; ++i, more = 1u) {
@@ -230,10 +233,16 @@ __device__ __forceinline__ void stream_gemm(const StreamPlan& sp, StreamShared& 
             const int b = seg & 1;
             if (!__all_sync(kFull, mbar_wait(smem_addr(&sh.acc_full[b]), (seg >> 1) & 1, abort_flag))) break;      // warp-uniform: tcgen05.ld is warp-wide
             tc_fence_after();
-            const uint32_t taddr = tmem + static_cast<uint32_t>(b * 2 * sp.ntok) + (static_cast<uint32_t>(q * 32) << 16);
+            const uint32_t taddr = tmem + static_cast<uint32_t>(b * sp.xrows) + (static_cast<uint32_t>(q * 32) << 16);
             for (int n0 = 0; n0 < sp.ntok && q * 32 < sp.rows; n0 += 16) {
                 float v[16];
-                tmem_ld16_sum(taddr + n0, taddr + sp.ntok + n0, v);
+                if (kFew) {
+                    tmem_ld16(taddr, v);
+#pragma unroll
+                    for (int i = 0; i < 16; ++i) v[i] = i < 4 ? v[i] + (v[i + 4] + v[i + 8]) : 0.f;
+                } else {
+                    tmem_ld16_sum(taddr + n0, taddr + sp.ntok + n0, v);
+                }
                 epi(tile, len == sp.call, q * 32 + lane, n0, v);
             }
             tc_fence_before();
@@ -255,6 +264,14 @@ __device__ __forceinline__ void stream_gemm(const StreamPlan& sp, StreamShared& 
 __device__ __forceinline__ void split_pair(float a, float b, unsigned& hi, unsigned& lo) {
     hi = pack2_bf16(a, b);
     lo = pack2_bf16(a - __uint_as_float(hi << 16), b - __uint_as_float(hi & 0xffff0000u));
+}
+
+// The three bf16 terms of an fp32 value pair: x = hi + mid + lo.
+__device__ __forceinline__ void split_pair3(float a, float b, unsigned& hi, unsigned& mid, unsigned& lo) {
+    hi = pack2_bf16(a, b);
+    const float ra = a - __uint_as_float(hi << 16), rb = b - __uint_as_float(hi & 0xffff0000u);
+    mid = pack2_bf16(ra, rb);
+    lo = pack2_bf16(ra - __uint_as_float(mid << 16), rb - __uint_as_float(mid & 0xffff0000u));
 }
 
 }  // namespace tc
