@@ -97,7 +97,7 @@ typedef struct spark_ctx spark_ctx;
 
 /* Bytes of workspace a context needs so that every call with batch <= max_batch,
  * d_ff <= max_dff, cache capacity <= max_cap, n_q query heads of head_dim hd and model
- * width <= max_d fits.  Pure host arithmetic. */
+ * width <= max_d fits, and for max_batch >= 32 a span of a prompt (spark_prefill).  Pure host arithmetic. */
 size_t spark_workspace_bytes(int64_t max_batch, int64_t max_dff, int64_t max_cap, int64_t n_q,
                              int64_t hd, int64_t max_d);
 
@@ -202,9 +202,10 @@ int spark_stat_select(spark_ctx* ctx, const float* x, int64_t rows, int64_t n, i
  * token with its own threshold and active set; weight rows are loaded once per call for the
  * union of the tokens' active sets (Appendix B).  Chunks of 5 to 64 tokens with bf16 weights, where
  * that union covers most rows, read every row instead and run the three products as GEMMs on the
- * tensor cores (same results; SPARK_DENSE_LOADS changes nothing there); this needs d % 256 == 0,
- * r % 64 == 0, d_ff % 128 == 0 and a workspace sized by spark_workspace_bytes for max_batch >= 5,
- * max_dff >= d_ff and max_d >= d -- any other call with 5..64 tokens takes the union-gather kernels.
+ * tensor cores (same results; SPARK_DENSE_LOADS changes nothing there); this needs r, d - r and d_ff
+ * of 64 and more, d_ff % 8 == 0 and <= 256 per SM, and a workspace sized by spark_workspace_bytes for
+ * max_batch >= 5, max_dff >= d_ff and max_d >= d -- any other call with 5..64 tokens takes the
+ * union-gather kernels.
  *   x [B][d] fp32;  K1t[d_ff][r], K2t[d_ff][d-r], Vt[d_ff][d] of dtype wdtype
  *   flags: SPARK_GELU_TANH or SPARK_GELU_ERF, optionally | SPARK_DENSE_LOADS
  *   y     [B][d]     fp32 (overwritten)
@@ -352,9 +353,9 @@ typedef struct spark_kv_cache {
  * undefined after the call.  h [B][d] fp32 is updated in place.  1 <= B <= 64.
  * Four kernels are enqueued for B <= 4: QKV projection with position encoding and cache
  * append, attention, output projection, FFN.  For B >= 5 the position encoding and the append follow the projection as a
- * kernel of their own, and where the shapes allow (see spark_ffn_decode; projections: inputs % 64 == 0, outputs % 128 == 0)
- * the projections and the FFN run as tensor-core GEMMs of two and four kernels each, and the attention of a chunk
- * (SPARK_SHARED_CACHE, B >= 16) as three: up to thirteen kernels per call. */
+ * kernel of their own, and where the shapes allow (see spark_ffn_decode; projections of 2 and more tokens: 64 inputs and
+ * more) the projections run as tensor-core GEMMs of two kernels each, the FFN as one (four for a small model), and the
+ * attention of a chunk (SPARK_SHARED_CACHE, B >= 16) as three: up to thirteen kernels per call. */
 int spark_layer_decode(spark_ctx* ctx, const spark_layer_weights* w, const spark_layer_cfg* cfg,
                        const spark_kv_cache* cache, const int32_t* ctx_len, float* h, int64_t B,
                        float* scratch, void* stream);
@@ -374,7 +375,10 @@ int spark_stack_decode(spark_ctx* ctx, const spark_layer_weights* w, const spark
  * the rows before it and to itself, later chunks seeing earlier ones through the caches -- what decoding the prompt token by token
  * gives.  w, cfg, cache: HOST arrays of n_layers structs; every cfg must carry SPARK_SHARED_CACHE (caches [n_kv][cap][.]) and
  * cap >= start + n_tokens.  len_buf: caller-owned DEVICE buffer of `chunk` int32 (the library writes each chunk's lengths there);
- * scratch as for spark_layer_decode with B = chunk.  The call only enqueues: one tiny kernel plus n_layers layer calls per chunk. */
+ * scratch as for spark_layer_decode with B = chunk.  The call only enqueues.  Several chunks go through the layers as one span of up
+ * to 1024 tokens where the workspace holds it (spark_workspace_bytes for max_batch >= 32 leaves room), the prompt has more than 64
+ * tokens, widths are multiples of 8 and spark_set_chunk_dense is not 0: the results are the same up to the order of floating-point
+ * reductions.  Otherwise one tiny kernel plus n_layers layer calls per chunk. */
 int spark_prefill(spark_ctx* ctx, const spark_layer_weights* w, const spark_layer_cfg* cfg, const spark_kv_cache* cache,
                   int64_t n_layers, float* h, int64_t n_tokens, int64_t start, int64_t chunk, int32_t* len_buf, float* scratch,
                   void* stream);
@@ -386,7 +390,8 @@ int spark_prefill(spark_ctx* ctx, const spark_layer_weights* w, const spark_laye
  * device (kernels that run at the same time must not share a workspace), scratch areas like spark_prefill's, and streams;
  * len_buf: n_inflight * chunk int32.  The call forks from streams[0] and joins back into it: work queued there before the call
  * is seen by all, work queued after it sees all of the prefill.  Creates and destroys n_inflight * (n_layers + 1) + 1 events
- * (no device memory).  Results equal spark_prefill's up to the order of floating-point reductions. */
+ * (no device memory).  Where spark_prefill would take spans (its note), they run on the first context and stream and nothing is in
+ * flight beside them.  Results equal spark_prefill's up to the order of floating-point reductions. */
 int spark_prefill_pipelined(spark_ctx* const* ctxs, float* const* scratches, void* const* streams, int64_t n_inflight,
                             const spark_layer_weights* w, const spark_layer_cfg* cfg, const spark_kv_cache* cache,
                             int64_t n_layers, float* h, int64_t n_tokens, int64_t start, int64_t chunk, int32_t* len_buf);

@@ -200,3 +200,14 @@ def test_argument_errors(ctx):
         assert e.value.status == code, bad
     call()
     torch.cuda.synchronize()
+
+
+@pytest.mark.parametrize("B,n_q,n_kv,hd,r,cap,k_attn", [(3, 4, 2, 256, 128, 32768, 256), (80, 4, 2, 64, 32, 120, 20), (5, 8, 1, 64, 32, 2500, 100), (160, 2, 2, 64, 32, 9, 3)])
+def test_blocks_that_span_segments(B, n_q, n_kv, hd, r, cap, k_attn):
+    # the flat cut: blocks with two pieces, half of the warps each (long and short ones, one and more warps per head), and with more than two
+    lens = [max(1, cap - (7 * b) % max(1, (2 * cap) // 3)) for b in range(B)]
+    a = synth.attn_inputs(B, n_q, n_kv, hd, r, cap, lens, "bf16", seed=B)
+    c = S.SparkContext(0, max_batch=B, max_cap=cap, n_q=n_q, hd=hd)
+    compare(a, run_attn(c, a, k_attn), k_attn, seqs=range(0, B, max(1, B // 12)))
+    assert c.device_status() == S.SPARK_OK
+    c.close()

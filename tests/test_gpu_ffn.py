@@ -99,6 +99,19 @@ def test_token_chunks_on_the_tensor_cores(ctx, d, d_ff, r, k, B, form):
     assert np.array_equal(again[1], out[1])
 
 
+@pytest.mark.parametrize("d,d_ff,r,k,B", [(256, 1000, 72, 80, 5), (256, 1000, 72, 80, 16), (256, 1000, 72, 80, 17), (136, 4104, 64, 300, 16), (136, 64, 72, 5, 64),
+                                         (1024, 4104, 512, 328, 9), (264, 18944, 136, 1500, 33), (264, 18952, 136, 1500, 64), (2304, 9224, 1024, 737, 48)])
+def test_tiles_of_the_chunk_kernels(ctx, d, d_ff, r, k, B):
+    # widths and neuron counts that divide no tile, a last tile of few neurons, one neuron tile per block and two (from 18945
+    # neurons on 148 SMs), the chain of small shapes and the one kernel on both sides of 16 tokens and of 16 MB of weights
+    p = synth.ffn_inputs(d, d_ff, r, k, B, "bf16", seed=d_ff + B)
+    w = upload(p)
+    out = run_ffn(ctx, p, weights=w)
+    assert compare(p, out) < 5e-3
+    again = run_ffn(ctx, p, weights=w, want_idx=False)
+    np.testing.assert_allclose(again[0], out[0], rtol=0, atol=1e-5 * parity.rms(out[0]))
+
+
 def test_gemma2_9b_shape_bf16(ctx):
     p = synth.ffn_inputs(3584, 14336, 1792, 1147, 2, "bf16", seed=1)
     compare(p, run_ffn(ctx, p))

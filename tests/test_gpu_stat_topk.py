@@ -177,3 +177,30 @@ def test_rows_held_on_chip_by_a_persistent_block(ctx, n, k, rows):
     else:
         assert np.all(np.isneginf(theta)) and np.all(count == n)
     compare_rows(X, k, S.SPARK_FILL_ZERO, out, rows=[0, 1, 147, 148, 149, rows - 1])
+
+
+# the register kernel (a warp to sixteen per row; to 8192 values always, lists of few rows to 65536 in clusters), the row kernel with
+# and without lists, on both sides of each limit; 3 %, 10 % and 30 % kept cross the line between staged and voted lists
+@pytest.mark.parametrize("frac", [0.03, 0.1, 0.3])
+@pytest.mark.parametrize("rows,n", [(5, 2), (33, 1023), (3, 1025), (4, 4096), (3, 8191), (3, 8193), (2, 16384), (200, 16385), (40, 28289), (3, 65536)])
+def test_each_output_alone_at_the_limits_of_the_kernels(ctx, rows, n, frac):
+    X = synth.rows_f32("normal", rows, n, seed=n) * 2.0 - 0.4
+    k = max(1, int(frac * n))
+    check = range(0, rows, max(1, rows // 5))
+    lists = run_topk(ctx, X, k, dense=False)
+    compare_rows(X, k, S.SPARK_FILL_ZERO, lists, rows=check)
+    ld = (n + 3) // 4 * 4
+    xd = torch.zeros((rows, ld), device="cuda")
+    xd[:, :n] = torch.from_numpy(X).cuda()
+    for dense in (False, True):
+        theta, count = torch.full((rows,), 123.0, device="cuda"), torch.full((rows,), -1, dtype=torch.int32, device="cuda")
+        yd = torch.full((rows, ld), float("nan"), device="cuda") if dense else None
+        S.spark_stat_topk(ctx, xd, rows, n, ld, k, S.SPARK_FILL_ZERO, theta, count, None, None, 0, yd)
+        th, c = theta.cpu().numpy(), count.cpu().numpy()
+        for i in check:
+            ref, _, _ = O.stat_topk(X[i], k, "zero")
+            parity.check_theta(th[i], ref, O.mean_std(X[i])[1], f"row {i}")
+        above = X > th[:, None]
+        assert np.array_equal(c, above.sum(axis=1))
+        if dense:      # one fp32 subtraction per kept value
+            assert np.array_equal(yd.cpu().numpy()[:, :n], np.where(above, X - th[:, None], np.float32(0)))
