@@ -543,9 +543,9 @@ int ffn_tc_launch(spark_ctx* ctx, FfnParams& f, cudaStream_t stream) {
         !make_map(&m_x1, p.g.xs, 2 * p.ntok, r, d, 2 * p.ntok, false) || !make_map(&m_x2, p.g.xs + r, 2 * p.ntok, d - r, d, 2 * p.ntok, false) ||
         !make_map(&m_v, f.Vt, d_ff, d, d, kChunk, true) || !make_map(&m_u, p.g.us, 2 * p.ntok, d_ff, d_ff, 2 * p.ntok, false))
         return SPARK_ERR_WORKSPACE;
-    // At least the share of an SM's shared memory that its columns are of tensor memory: blocks that hold columns while they wait for
-    // other blocks then never share an SM with so many of their kind that one waits for columns.
-    const size_t want = static_cast<size_t>(p.stages) * p.stage_bytes + 1024, least = (static_cast<size_t>(ctx->max_smem_optin) + 1024) * p.tmem_cols / 512;
+    // Blocks that hold tensor memory while they wait for other blocks: no more of their kind may share an SM than there are columns
+    // for, so each takes at least the shared memory that keeps the next one out.
+    const size_t want = static_cast<size_t>(p.stages) * p.stage_bytes + 1024, least = (static_cast<size_t>(ctx->max_smem_optin) + 1024) / (512 / p.tmem_cols + 1);
     const void* kern = reinterpret_cast<const void*>(ffn_tc_kernel);
     if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, limit) != cudaSuccess) return SPARK_ERR_CUDA;
     void* args[] = {&p, &m_k1, &m_x1, &m_k2, &m_x2, &m_v, &m_u};

@@ -187,9 +187,9 @@ def test_each_output_alone_at_the_limits_of_the_kernels(ctx, rows, n, frac):
     X = synth.rows_f32("normal", rows, n, seed=n) * 2.0 - 0.4
     k = max(1, int(frac * n))
     check = range(0, rows, max(1, rows // 5))
-    lists = run_topk(ctx, X, k, dense=False)
-    compare_rows(X, k, S.SPARK_FILL_ZERO, lists, rows=check)
     ld = (n + 3) // 4 * 4
+    lists = run_topk(ctx, X, k, dense=False, ld=ld)
+    compare_rows(X, k, S.SPARK_FILL_ZERO, lists, rows=check)
     xd = torch.zeros((rows, ld), device="cuda")
     xd[:, :n] = torch.from_numpy(X).cuda()
     for dense in (False, True):
