@@ -254,7 +254,7 @@ def measure_stack(torch, S, dist, dev, rank, world, shape_name, B, ctx_len, n_la
     h_host_out = torch.empty_like(h_host_in).pin_memory()
     # QKV (+ rotary, append: a kernel of their own for B >= 5), attention, output projection, FFN; for B >= 5 the projections
     # are two kernels each (prep, tcgen05 GEMM) and the FFN four (prep, scores, activation, output)
-    kernels_per_layer = 4 if B <= 4 else 10
+    kernels_per_layer = 4 if B == 1 else (5 if B <= 4 else 7)
 
     def stack(which):
         for lay in layers:
@@ -386,7 +386,7 @@ def measure_stack(torch, S, dist, dev, rank, world, shape_name, B, ctx_len, n_la
                                    shape.k_ff, 0, y, None, None, None)
         cl.fill_(ctx_len + 1)
         rows_read = union if B <= 4 else shape.d_ff
-        out["ffn"] = entry(("ffn1_kernel" if B == 1 else "ffn_few_kernel" if B <= 4 else "ffn_tc_{prep,scores,act,out}_kernel") +
+        out["ffn"] = entry(("ffn1_kernel" if B == 1 else "ffn_few_kernel" if B <= 4 else "ffn_tc_kernel") +
                            " (spark_ffn_decode)", loop_us(ffn_calls), shape.d_ff * shape.r_ff * 2 + rows_read * (2 * d - shape.r_ff) * 2)
 
         qa = torch.randn(B, shape.n_q, hd, device=dev, generator=gen) / (hd ** 0.5)
