@@ -252,8 +252,8 @@ def measure_stack(torch, S, dist, dev, rank, world, shape_name, B, ctx_len, n_la
     scratch = torch.empty(S.layer_scratch_floats(dict(n_q=shape.n_q, n_kv=shape.n_kv, hd=hd, d=d), B), device=dev)
     h_host_in = h_init.cpu().pin_memory()
     h_host_out = torch.empty_like(h_host_in).pin_memory()
-    # QKV (+ rotary, append: a kernel of their own for B >= 5), attention, output projection, FFN; for B >= 5 the projections
-    # are two kernels each (prep, tcgen05 GEMM) and the FFN four (prep, scores, activation, output)
+    # QKV (+ rotary, append: a kernel of their own for B >= 5), attention, output projection, FFN; from two sequences on
+    # the output projection, from five on both projections are two kernels each (prep, tcgen05 GEMM)
     kernels_per_layer = 4 if B == 1 else (5 if B <= 4 else 7)
 
     def stack(which):
