@@ -658,9 +658,10 @@ extern "C" int spark_layer_decode(spark_ctx* ctx, const spark_layer_weights* w, 
     int rc;
     const int tbq = B == 1 ? 1 : (B <= 4 ? 4 : 16);
     const size_t smem_q = static_cast<size_t>(tbq) * cfg->d * 4;
-    // up to four tokens: projection, rotary encoding and cache append in one kernel; more: the tensor-core GEMV,
-    // then a small kernel for the rotary encoding and the append
-    if (B <= 4 && (cfg->d & 7) == 0 && smem_q <= static_cast<size_t>(ctx->max_smem_optin - 1024) && nqkv / 2 >= 1 &&
+    // one token: projection, rotary encoding and cache append in one kernel; more: the tensor-core projection, then a small kernel for the
+    // rotary encoding and the append (the fused kernel on the plain ALUs took longer than both from two tokens on: layers of the 2B shape
+    // at batch 2 49.0 -> 44.2 us, at batch 4 60.1 -> 54.9, of the 9B shape at batch 2 83.9 -> 74.2, batch 4 106.9 -> 95.3)
+    if (B == 1 && (cfg->d & 7) == 0 && smem_q <= static_cast<size_t>(ctx->max_smem_optin - 1024) && nqkv / 2 >= 1 &&
         aligned16(w->Wqkv) && aligned16(w->norm1)) {
         if (k1_f8) { rp.k1f32 = qkv; rp.k1f32_sb = cfg->n_kv * cfg->r_attn; rp.k1f32_sg = cfg->r_attn; }      // the projection buffer is free here
         QkvRopeParams qp;
