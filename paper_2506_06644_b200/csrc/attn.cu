@@ -134,6 +134,7 @@ __global__ void __launch_bounds__(kThreads, 1) attn_kernel(const AttnParams p) {
     __shared__ double red[kWarps][GQ][2];
     __shared__ float redm[kWarps][GQ];
     __shared__ float theta_s[2][GQ], smax_s[2][GQ];            // of the pieces in hand
+    __shared__ double z_s[2];                                  // quantiles of the block's first two pieces
     __shared__ int s_last[2], s_fail, s_aligned;
     __shared__ __align__(16) unsigned char q8[sizeof(K1T) == 1 ? 8 * kQ8Stride : (M16 ? 8 * kQ16Stride : 16)];   // tensor-core pass 1: query terms
     __shared__ float qsc[8];                                                             //   and their scales, per column
@@ -330,6 +331,9 @@ __global__ void __launch_bounds__(kThreads, 1) attn_kernel(const AttnParams p) {
             const int off = static_cast<int>(f - f0) - tb;           // score slot of token t: off + t
             float* qs = qs0 + (ord & 1) * GQ * hd;
             for (int i = tid; i < GQ * hd; i += kThreads) qs[i] = p.q[(static_cast<int64_t>(b) * p.n_q + g * GQ) * hd + i];
+            // the quantile of the threshold under the first rows' latency (a double-precision inverse takes a microsecond)
+            if (tid == kThreads - 1 && ord < 2)
+                z_s[ord] = p.k_attn >= L ? 0.0 : (p.zs != nullptr ? p.zs[b] : -normcdfinv(static_cast<double>(p.k_attn) / static_cast<double>(L)));
             if (tb == 0 && p.count != nullptr && tid < GQ) p.count[b * p.n_q + g * GQ + tid] = 0;
             if (tb == 0) {      // the segment's first piece clears the heads' accumulators before it arrives
                 float* ob = p.o + (static_cast<int64_t>(b) * p.n_q + g * GQ) * hd;
@@ -668,8 +672,8 @@ __global__ void __launch_bounds__(kThreads, 1) attn_kernel(const AttnParams p) {
             if (wl < GQ) {          // theta of this head once every piece of the segment has arrived
                 double sa, sq, z = 0.0;
                 float smax;
-                // the quantile under the wait for the other blocks (a double-precision inverse takes a microsecond)
-                if (!c.ident) z = p.zs != nullptr ? p.zs[c.b] : -normcdfinv(static_cast<double>(p.k_attn) / static_cast<double>(c.L));
+                if (ord == 0) z = z_s[wz];
+                else if (!c.ident) z = p.zs != nullptr ? p.zs[c.b] : -normcdfinv(static_cast<double>(p.k_attn) / static_cast<double>(c.L));
                 const bool ok = cells_wait_max_w<kAttnWays>(cells + static_cast<size_t>(c.b * p.n_q + c.g * GQ + wl) * kAttnWays,
                                                             static_cast<unsigned>(c.npieces), sa, sq, smax, p.hdr);
                 if (lane == 0) {
